@@ -204,6 +204,22 @@ pconv_status pconv_forward_ws(const pconv_handle* h, const void* x_dev, const fl
                               size_t ws_bytes, void* stream);
 
 /*
+ * pconv_scratch_bytes / pconv_forward_scratch -- pconv_forward_ws with room for the input in the layout
+ * the tensor cores read.  With it a layer that takes the dense tensor-core kernel is run as two
+ * launches: one lays the input out (once, instead of every thread block converting what it needs), one
+ * multiplies.  The result is the same up to summation order.
+ *
+ *  bytes        receives the size for this handle and input shape (0 = never used).
+ *  ws_dev       as for pconv_forward_ws (may be NULL).
+ *  scratch_dev  DEVICE buffer, 256-byte aligned, or NULL (= pconv_forward_ws); contents irrelevant
+ *               before and after.  Forwards that share it must not overlap in time.
+ */
+pconv_status pconv_scratch_bytes(const pconv_handle* h, int n, int h_in, int w_in, size_t* bytes);
+pconv_status pconv_forward_scratch(const pconv_handle* h, const void* x_dev, const float* bias_dev,
+                                   void* y_dev, int n, int h_in, int w_in, unsigned flags, void* ws_dev,
+                                   size_t ws_bytes, void* scratch_dev, size_t scratch_bytes, void* stream);
+
+/*
  * pconv_forward_static_ws -- pconv_forward_ws for callers that cannot allocate device memory.
  * (The paper has no counterpart: this entry point exists for integration, not for the method.)
  *

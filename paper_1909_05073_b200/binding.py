@@ -6,6 +6,7 @@ raises.  torch is used for device memory and streams only.
 """
 import ctypes
 import os
+import threading
 
 import numpy as np
 
@@ -24,7 +25,7 @@ STATUS_NAMES = ["PCONV_OK", "PCONV_ERR_NULL", "PCONV_ERR_SHAPE", "PCONV_ERR_PATT
                 "PCONV_ERR_ALIGN", "PCONV_ERR_ALLOC", "PCONV_ERR_CUDA",
                 "PCONV_ERR_DEVICE_TIMEOUT", "PCONV_ERR_WORKSPACE"]
 
-EXPORTS = ["pconv_pack", "pconv_forward", "pconv_forward_ws", "pconv_forward_static_ws", "pconv_workspace_bytes", "pconv_plan", "pconv_plan_shape",
+EXPORTS = ["pconv_pack", "pconv_forward", "pconv_forward_ws", "pconv_forward_static_ws", "pconv_forward_scratch", "pconv_scratch_bytes", "pconv_workspace_bytes", "pconv_plan", "pconv_plan_shape",
            "pconv_free", "pconv_maxpool2x2", "pconv_unpack",
            "pconv_stats", "pconv_filter_order", "pconv_device_status", "pconv_status_str",
            "pconv_stack_create", "pconv_stack_out_shape", "pconv_stack_forward",
@@ -76,6 +77,8 @@ def load(path):
     L.pconv_forward.argtypes = [vp, vp, vp, vp, ci, ci, ci, cu, vp]
     L.pconv_forward_ws.argtypes = [vp, vp, vp, vp, ci, ci, ci, cu, vp, ctypes.c_size_t, vp]
     L.pconv_forward_static_ws.argtypes = [vp, vp, vp, vp, ci, ci, ci, cu, vp]
+    L.pconv_forward_scratch.argtypes = [vp, vp, vp, vp, ci, ci, ci, cu, vp, ctypes.c_size_t, vp, ctypes.c_size_t, vp]
+    L.pconv_scratch_bytes.argtypes = [vp, ci, ci, ci, ctypes.POINTER(ctypes.c_size_t)]
     L.pconv_workspace_bytes.argtypes = [vp, ci, ci, ci, ctypes.POINTER(ctypes.c_size_t)]
     L.pconv_plan.argtypes = [vp, ci, ci, ci, cu, ci, ctypes.POINTER(Plan)]
     L.pconv_plan_shape.argtypes = [ci, ci, ctypes.c_longlong, ci, ci, ci, ci, ci, ci, cu, ci,
@@ -132,10 +135,11 @@ def _check(status, what, detail=None):
 
 
 def _stream_ptr(stream=None):
+    """A stream (default: torch's current one) as the integer the library takes."""
     import torch
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream.cuda_stream
 
 
 def _storage_of(t):
@@ -223,9 +227,16 @@ def pconv_workspace_bytes(handle, n, h, w):
     return int(b.value)
 
 
-def pconv_forward(handle, x, bias, y, flags=0, stream=None, workspace=None):
+def pconv_scratch_bytes(handle, n, h, w):
+    b = ctypes.c_size_t(0)
+    _check(lib().pconv_scratch_bytes(handle, n, h, w, ctypes.byref(b)), "pconv_scratch_bytes")
+    return int(b.value)
+
+
+def pconv_forward(handle, x, bias, y, flags=0, stream=None, workspace=None, scratch=None):
     """x, y: CUDA torch tensors (NCHW, contiguous); bias: CUDA fp32 tensor or None;
-    workspace: zeroed CUDA uint8 tensor from pconv_workspace_bytes, or None."""
+    workspace: zeroed CUDA uint8 tensor from pconv_workspace_bytes, or None; scratch: CUDA uint8
+    tensor of pconv_scratch_bytes, contents irrelevant, or None."""
     if not (x.is_cuda and y.is_cuda and x.is_contiguous() and y.is_contiguous()):
         raise ValueError("x and y must be contiguous CUDA tensors")
     n, _, h, w = x.shape
@@ -233,16 +244,15 @@ def pconv_forward(handle, x, bias, y, flags=0, stream=None, workspace=None):
     if bias is not None:
         if not (bias.is_cuda and bias.is_contiguous()) or bias.dtype.itemsize != 4:
             raise ValueError("bias must be a contiguous CUDA float32 tensor")
-        bp = ctypes.c_void_p(bias.data_ptr())
-    if workspace is not None:
-        st = lib().pconv_forward_ws(handle, ctypes.c_void_p(x.data_ptr()), bp,
-                                    ctypes.c_void_p(y.data_ptr()), n, h, w, int(flags),
-                                    ctypes.c_void_p(workspace.data_ptr()), workspace.numel(),
-                                    _stream_ptr(stream))
+        bp = bias.data_ptr()
+    # (pointers as plain integers: the declared argument types convert them)
+    if scratch is not None or workspace is not None:
+        st = lib().pconv_forward_scratch(
+            handle, x.data_ptr(), bp, y.data_ptr(), n, h, w, int(flags),
+            None if workspace is None else workspace.data_ptr(), 0 if workspace is None else workspace.numel(),
+            None if scratch is None else scratch.data_ptr(), 0 if scratch is None else scratch.numel(), _stream_ptr(stream))
     else:
-        st = lib().pconv_forward(handle, ctypes.c_void_p(x.data_ptr()), bp,
-                                 ctypes.c_void_p(y.data_ptr()), n, h, w, int(flags),
-                                 _stream_ptr(stream))
+        st = lib().pconv_forward(handle, x.data_ptr(), bp, y.data_ptr(), n, h, w, int(flags), _stream_ptr(stream))
     _check(st, "pconv_forward")
 
 
@@ -303,6 +313,8 @@ class Layer:
         import torch
         self.handle = pconv_pack(w_oihw, patterns, stride, storage, STRICT4 if strict4 else 0)
         self.stride, self.storage = stride, storage
+        self._ws, self._ws_need = None, {}          # sizes by input shape: asked for once
+        self._scratch, self._scratch_need = {}, {}
         self.c_out, self.c_in = int(w_oihw.shape[0]), int(w_oihw.shape[1])
         self.bias = None
         if bias is not None:
@@ -314,25 +326,49 @@ class Layer:
 
     def workspace(self, x_shape):
         """A zeroed workspace for inputs of this shape (cached), or None if never needed."""
-        import torch
-        n, _, h, w = x_shape
-        need = pconv_workspace_bytes(self.handle, n, h, w)
+        x_shape = tuple(x_shape)
+        need = self._ws_need.get(x_shape)
+        if need is None:
+            n, _, h, w = x_shape
+            need = self._ws_need[x_shape] = pconv_workspace_bytes(self.handle, n, h, w)
         if need == 0:
             return None
-        ws = getattr(self, "_ws", None)
+        ws = self._ws
         if ws is None or ws.numel() < need:
+            import torch
             ws = self._ws = torch.zeros(need, dtype=torch.uint8, device="cuda")
         return ws
 
+    def scratch(self, x_shape):
+        """Scratch memory for inputs of this shape, or None if never used: one buffer for each
+        (thread, stream) that calls, so that concurrent forwards of a layer do not share one; the last
+        few are kept."""
+        x_shape = tuple(x_shape)
+        need = self._scratch_need.get(x_shape)
+        if need is None:
+            n, _, h, w = x_shape
+            need = self._scratch_need[x_shape] = pconv_scratch_bytes(self.handle, n, h, w)
+        if need == 0:
+            return None
+        who = (threading.get_ident(), _stream_ptr())
+        buf = self._scratch.get(who)
+        if buf is None or buf.numel() < need:
+            import torch
+            if len(self._scratch) >= 8:
+                self._scratch.pop(next(iter(self._scratch)), None)
+            buf = self._scratch[who] = torch.empty(need, dtype=torch.uint8, device="cuda")
+        return buf
+
     def forward(self, x, relu=True, kernel=0, out=None, split=False, pool=False):
-        import torch
         if out is None:
+            import torch
             n, c, h, w = self.out_shape(x.shape)
             shape = (n, c, h // 2, w // 2) if pool else (n, c, h, w)
             out = torch.empty(shape, dtype=x.dtype, device=x.device)
         ws = self.workspace(x.shape) if split else None
         pconv_forward(self.handle, x, self.bias, out,
-                      (RELU if relu else 0) | (POOL2X2 if pool else 0) | kernel, workspace=ws)
+                      (RELU if relu else 0) | (POOL2X2 if pool else 0) | kernel, workspace=ws,
+                      scratch=self.scratch(x.shape) if kernel == 0 else None)
         return out
 
     def stats(self):
@@ -374,8 +410,7 @@ class Stack:
         self.in_shape = (n, self.layers[0].c_in, h, w)
 
     def forward(self, x, y, stream=None):
-        _check(lib().pconv_stack_forward(self.ptr, ctypes.c_void_p(x.data_ptr()),
-                                         ctypes.c_void_p(y.data_ptr()), _stream_ptr(stream)),
+        _check(lib().pconv_stack_forward(self.ptr, x.data_ptr(), y.data_ptr(), _stream_ptr(stream)),
                "pconv_stack_forward")
 
     def capture(self, x, y, stream):

@@ -1,4 +1,5 @@
 // C ABI entry points: argument checks, kernel selection, layer stacks.
+#include <algorithm>
 #include <cstring>
 #include <cstdlib>
 #include <mutex>
@@ -54,10 +55,23 @@ static int rows_mode(unsigned flags) {
   return ((flags & PCONV_ROWS8) ? 8 : (flags & PCONV_ROWS4) ? 4 : 0) | ((flags & PCONV_STAGE_BULK) ? pconv::kPinBulk : 0);
 }
 
+// fp16 storage, stride 1 and a batch that gives a fair part of the device 128-position tiles of its own:
+// the case in which a default forward is, without any estimate, the pinned tensor-core kernel.  The
+// zero-inserted contraction at a fifth of the tensor peak must be cheaper than the surviving
+// multiply-adds at a fifth of the FP32 peak.
+static bool batch_on_tensor_cores(const pconv::DeviceLayer& L, int n, int h, int w) {
+  if (L.storage != PCONV_F16 || L.stride != 1 || !dense_supported(L, n, h, w, false)) return false;
+  const double tiles = (double)n * (h + 1) * (w + 1) / 128.0 * ((L.dense_rows + 127) / 128);
+  if (tiles < device_sm_count() / 4) return false;
+  const double dense = 2.0 * 9.0 * (16.0 * ((L.c_in + 15) / 16)) * L.dense_rows, sparse = 8.0 * (double)L.n_kept;
+  return dense / (0.2 * 2250e12) < sparse / (0.2 * 74.45e12);
+}
+
 // Scratch a forward of this shape may use, whichever kernel takes it.  rmode: the rows per lane
-// the caller pins for the tiled kernel (0 = the planner's choice), -1 = whatever it may pin.
-static size_t workspace_need(const pconv::DeviceLayer& L, int n, int h_in, int w_in, int rmode) {
-  size_t need = tensor_workspace_bytes(L, n, h_in, w_in);
+// the caller pins for the tiled kernel (0 = the planner's choice), -1 = whatever it may pin.  The dense
+// kernel makes do with what it gets: `most_dense` bounds what it asks for.
+static size_t workspace_need(const pconv::DeviceLayer& L, int n, int h_in, int w_in, int rmode, size_t most_dense) {
+  size_t need = dense_workspace_bytes(L, n, h_in, w_in, most_dense);
   for (int r = 0; r <= 8; r += 4)
     for (int bulk = 0; bulk <= pconv::kPinBulk; bulk += pconv::kPinBulk) {
       if (rmode >= 0 && (r | bulk) != rmode) continue;
@@ -74,7 +88,7 @@ extern "C" pconv_status pconv_workspace_bytes(const pconv_handle* h, int n, int 
   // (whichever kernel a forward of this shape may take)
   *bytes = 0;
   if (n > 0) {
-    *bytes = workspace_need(h->d, n, h_in, w_in, -1);
+    *bytes = workspace_need(h->d, n, h_in, w_in, -1, pconv::kMaxSplitBytes);
   }
   return PCONV_OK;
 }
@@ -87,7 +101,7 @@ extern "C" pconv_status pconv_plan(const pconv_handle* h, int n, int h_in, int w
   if (!tiled_plan(h->d, n, h_in, w_in, (flags & PCONV_KERNEL_GENERIC_TAPS) != 0, with_workspace != 0,
                   rows_mode(flags), plan))
     return PCONV_ERR_UNSUPPORTED;
-  plan->tensor_path = tensor_preferred(h->d, n, h_in, w_in) ? 1 : 0;
+  plan->tensor_path = batch_on_tensor_cores(h->d, n, h_in, w_in) ? 1 : 0;
   return PCONV_OK;
 }
 
@@ -126,18 +140,34 @@ extern "C" pconv_status pconv_forward(const pconv_handle* h, const void* x, cons
 // abandoned wait there instead of in the handle's own status block (a stack collects the status
 // of all its layers in one word).
 static pconv_status forward_impl(const pconv_handle* h, const void* x, const float* bias, void* y,
-                                 int n, int h_in, int w_in, unsigned flags, void* ws,
-                                 size_t ws_bytes, void* stream_v, int* status_dev);
+                                 int n, int h_in, int w_in, unsigned flags, void* ws, size_t ws_bytes, void* scratch,
+                                 size_t scratch_bytes, void* stream_v, int* status_dev);
 
 extern "C" pconv_status pconv_forward_ws(const pconv_handle* h, const void* x, const float* bias,
                                          void* y, int n, int h_in, int w_in, unsigned flags,
                                          void* ws, size_t ws_bytes, void* stream_v) {
-  return forward_impl(h, x, bias, y, n, h_in, w_in, flags, ws, ws_bytes, stream_v, nullptr);
+  return forward_impl(h, x, bias, y, n, h_in, w_in, flags, ws, ws_bytes, nullptr, 0, stream_v, nullptr);
+}
+
+extern "C" pconv_status pconv_scratch_bytes(const pconv_handle* h, int n, int h_in, int w_in, size_t* bytes) {
+  if (!h || !bytes) return PCONV_ERR_NULL;
+  if (n < 0 || h_in <= 0 || w_in <= 0) return PCONV_ERR_SHAPE;
+  *bytes = 0;
+  for (int pool = 0; n > 0 && pool < 2; ++pool)
+    *bytes = std::max(*bytes, dense_rows_bytes(h->d, n, h_in, w_in, pool != 0));
+  return PCONV_OK;
+}
+
+extern "C" pconv_status pconv_forward_scratch(const pconv_handle* h, const void* x, const float* bias, void* y, int n,
+                                              int h_in, int w_in, unsigned flags, void* ws, size_t ws_bytes,
+                                              void* scratch, size_t scratch_bytes, void* stream_v) {
+  if (scratch && ((uintptr_t)scratch & 255u)) return PCONV_ERR_ALIGN;
+  return forward_impl(h, x, bias, y, n, h_in, w_in, flags, ws, ws_bytes, scratch, scratch_bytes, stream_v, nullptr);
 }
 
 static pconv_status forward_impl(const pconv_handle* h, const void* x, const float* bias, void* y,
-                                 int n, int h_in, int w_in, unsigned flags, void* ws,
-                                 size_t ws_bytes, void* stream_v, int* status_dev) {
+                                 int n, int h_in, int w_in, unsigned flags, void* ws, size_t ws_bytes, void* scratch,
+                                 size_t scratch_bytes, void* stream_v, int* status_dev) {
   if (!h || !x || !y) return PCONV_ERR_NULL;
   if (n < 0 || h_in <= 0 || w_in <= 0) return PCONV_ERR_SHAPE;
   const unsigned known =
@@ -173,13 +203,25 @@ static pconv_status forward_impl(const pconv_handle* h, const void* x, const flo
   const bool pool = flags & PCONV_POOL2X2;
   const bool repro = flags & PCONV_REPRODUCIBLE;
   cudaError_t e;
-  if (pool && (sel == PCONV_KERNEL_SIMPLE || !tiled_supported(L, n, h_in, w_in)))
-    return PCONV_ERR_UNSUPPORTED;  // only the tiled kernels fuse the pool
-  if (sel == PCONV_KERNEL_TENSOR) {
-    if (pool || !tensor_supported(L, n, h_in, w_in)) return PCONV_ERR_UNSUPPORTED;
-    e = launch_tensor(L, x, bias, y, n, h_in, w_in, relu, repro ? nullptr : ws, ws_bytes, stream);
-  } else if (sel == 0 && !pool && tensor_preferred(L, n, h_in, w_in)) {
-    e = launch_tensor(L, x, bias, y, n, h_in, w_in, relu, repro ? nullptr : ws, ws_bytes, stream);
+  // nothing pinned: the dense tensor-core kernel where it is expected to be the faster one, on position
+  // rows staged in the caller's scratch memory if there is enough of it
+  void* dense_ws = repro ? nullptr : ws;
+  const size_t dense_ws_bytes = dense_ws ? ws_bytes : 0;
+  const size_t rows = scratch ? dense_rows_bytes(L, n, h_in, w_in, pool) : 0;
+  const DensePath path = dense_path(L, n, h_in, w_in, pool, rows > 0 && rows <= scratch_bytes ? kRowsStaged : kNoRows,
+                                    dense_ws_bytes);
+  const bool staged = path == kFromRows;
+  const bool dense = sel == 0 && rmode == 0 && !cluster &&
+                     (path != kNotDense || (!pool && batch_on_tensor_cores(L, n, h_in, w_in)));
+  if (pool && !dense && (sel == PCONV_KERNEL_SIMPLE || !tiled_supported(L, n, h_in, w_in)))
+    return PCONV_ERR_UNSUPPORTED;  // the plain kernel does not fuse the pool
+  if (dense || sel == PCONV_KERNEL_TENSOR) {
+    if (!dense && (pool || L.storage != PCONV_F16 || L.stride != 1 || !dense_supported(L, n, h_in, w_in, false)))
+      return PCONV_ERR_UNSUPPORTED;
+    e = staged ? launch_stage(L, x, scratch, n, h_in, w_in, pool, stream) : cudaSuccess;
+    if (e == cudaSuccess)
+      e = launch_dense(L, staged ? scratch : x, bias, y, n, h_in, w_in, relu, pool, staged, nullptr, dense_ws,
+                       dense_ws_bytes, stream);
   } else if (sel == PCONV_KERNEL_SIMPLE) {
     e = launch_simple(L, x, bias, y, n, h_in, w_in, relu, stream);
   } else if (sel == PCONV_KERNEL_TILED || sel == PCONV_KERNEL_GENERIC_TAPS) {
@@ -234,7 +276,7 @@ extern "C" pconv_status pconv_forward_static_ws(const pconv_handle* h, const voi
   if (!h || !x || !y) return PCONV_ERR_NULL;
   if (n < 0 || h_in <= 0 || w_in <= 0) return PCONV_ERR_SHAPE;
   if (n == 0) return PCONV_OK;
-  const size_t need = workspace_need(h->d, n, h_in, w_in, rows_mode(flags));
+  const size_t need = workspace_need(h->d, n, h_in, w_in, rows_mode(flags), PCONV_STATIC_WS_BYTES);
   if (need > (size_t)PCONV_STATIC_WS_BYTES) return PCONV_ERR_WORKSPACE;
   if (need == 0)  // this shape is never split: no scratch involved
     return pconv_forward_ws(h, x, bias, y, n, h_in, w_in, flags, nullptr, 0, stream_v);
@@ -287,7 +329,8 @@ extern "C" pconv_status pconv_trace_read(const pconv_handle* h, unsigned long lo
 }
 
 extern "C" pconv_status pconv_dev_withhold(int chunk, unsigned spin_limit) {
-  if (pconv::dev_set_withhold(chunk, spin_limit) != cudaSuccess) {
+  if (pconv::dev_set_withhold(chunk, spin_limit) != cudaSuccess ||
+      pconv::dense_set_withhold(chunk, spin_limit) != cudaSuccess) {
     cudaGetLastError();
     return PCONV_ERR_CUDA;
   }
@@ -336,6 +379,11 @@ struct pconv_stack {
     std::vector<void*> mid;    // outputs of the chain's inner layers (never reused inside the launch)
   };
   std::vector<Chain>* chains;
+  // layers that the dense kernel runs on position rows: rows[i] = layer i's input in that layout (its padding
+  // zero from the start: only real positions are ever written), or null where layer i reads NCHW
+  std::vector<void*>* rows;
+  void* rows_block;            // the one allocation behind them
+  std::vector<pconv::DensePath>* path;
   unsigned int* sync_dev;      // the chain kernel's two counters (zero between launches)
 };
 
@@ -355,6 +403,9 @@ extern "C" void pconv_stack_free(pconv_stack* s) {
     }
     delete s->chains;
   }
+  if (s->rows_block) cudaFree(s->rows_block);
+  delete s->rows;
+  delete s->path;
   if (s->sync_dev) cudaFree(s->sync_dev);
   if (s->status_dev) cudaFree(s->status_dev);
   if (s->status_host) cudaFreeHost(s->status_host);
@@ -383,7 +434,7 @@ static bool build_chains(pconv_stack* s) {
       hi[i] = ch;
       wi[i] = cw;
       ok[i] = pconv::chain_layer_ok(L, s->n, ch, cw, s->pool[i] != 0, nullptr) &&
-              !pconv::tensor_preferred(L, s->n, ch, cw);
+              !batch_on_tensor_cores(L, s->n, ch, cw);
       ch = (ch - 1) / L.stride + 1;
       cw = (cw - 1) / L.stride + 1;
       if (s->pool[i]) {
@@ -444,6 +495,58 @@ static bool build_chains(pconv_stack* s) {
   return true;
 }
 
+// Whether a pool that follows a layer of this input shape is fused into the layer's epilogue (a pinned
+// plain or tensor-core kernel has no pooled form: the plain max-pool kernel follows it).
+static bool fuses_pool(const pconv_stack* s, int i, int h, int w) {
+  if (s->flags & (PCONV_KERNEL_SIMPLE | PCONV_KERNEL_TENSOR)) return false;
+  return (*s->path)[i] != pconv::kNotDense || pconv::tiled_supported(s->layers[i]->d, s->n, h, w);
+}
+
+// Chooses the kernel of every layer that is not pinned or inside a chain, and gives those that run on
+// position rows their input buffer: the layer before writes it if it is a dense one too, else it is staged.
+static bool build_rows(pconv_stack* s) {
+  s->rows = new (std::nothrow) std::vector<void*>(s->n_layers, nullptr);
+  s->path = new (std::nothrow) std::vector<pconv::DensePath>(s->n_layers, pconv::kNotDense);
+  if (!s->rows || !s->path) return false;
+  const unsigned pinned = PCONV_KERNEL_SIMPLE | PCONV_KERNEL_TILED | PCONV_KERNEL_GENERIC_TAPS | PCONV_KERNEL_TENSOR |
+                          PCONV_ROWS4 | PCONV_ROWS8 | PCONV_CLUSTER | PCONV_STAGE_BULK;
+  if (s->flags & pinned) return true;
+  const size_t ws_bytes = (s->flags & PCONV_REPRODUCIBLE) ? 0 : s->ws_bytes;
+  std::vector<size_t> at(s->n_layers, 0);
+  size_t total = 0;
+  int ch = s->h, cw = s->w;
+  for (int i = 0; i < s->n_layers; ++i) {
+    const pconv::DeviceLayer& L = s->layers[i]->d;
+    bool chained = false;
+    for (const pconv_stack::Chain& c : *s->chains) chained = chained || (i >= c.begin && i < c.end);
+    const bool pool = s->pool[i] != 0;
+    if (!chained) {
+      const size_t bytes = pconv::dense_rows_bytes(L, s->n, ch, cw, pool);
+      const bool given = bytes > 0 && i > 0 && (*s->path)[i - 1] != pconv::kNotDense;
+      (*s->path)[i] = pconv::dense_path(L, s->n, ch, cw, pool,
+                                        given ? pconv::kRowsGiven : bytes > 0 ? pconv::kRowsStaged : pconv::kNoRows, ws_bytes);
+      if ((*s->path)[i] == pconv::kNotDense && batch_on_tensor_cores(L, s->n, ch, cw) &&
+          pconv::dense_supported(L, s->n, ch, cw, pool))
+        (*s->path)[i] = pconv::kFromNchw;
+      if ((*s->path)[i] == pconv::kFromRows) {
+        at[i] = total + 1;
+        total += (bytes + 255) & ~(size_t)255;
+      }
+    }
+    ch = (ch - 1) / L.stride + 1;
+    cw = (cw - 1) / L.stride + 1;
+    if (pool) {
+      ch /= 2;
+      cw /= 2;
+    }
+  }
+  if (total && (cudaMalloc(&s->rows_block, total) != cudaSuccess || cudaMemset(s->rows_block, 0, total) != cudaSuccess))
+    return false;
+  for (int i = 0; i < s->n_layers; ++i)
+    if (at[i]) (*s->rows)[i] = (char*)s->rows_block + at[i] - 1;
+  return true;
+}
+
 extern "C" pconv_status pconv_stack_create(const pconv_handle* const* layers,
                                            const float* const* bias_dev,
                                            const unsigned char* pool_after, int n_layers, int n,
@@ -481,7 +584,7 @@ extern "C" pconv_status pconv_stack_create(const pconv_handle* const* layers,
       pconv_stack_free(s);
       return PCONV_ERR_SHAPE;
     }
-    const size_t wsb = tiled_workspace_bytes(L, n, ch, cw, rows_mode(flags)), wsd = tensor_workspace_bytes(L, n, ch, cw);
+    const size_t wsb = tiled_workspace_bytes(L, n, ch, cw, rows_mode(flags)), wsd = dense_workspace_bytes(L, n, ch, cw, pconv::kMaxSplitBytes);
     if (wsb > s->ws_bytes) s->ws_bytes = wsb;
     if (wsd > s->ws_bytes) s->ws_bytes = wsd;
     ch = (ch - 1) / L.stride + 1;
@@ -511,7 +614,7 @@ extern "C" pconv_status pconv_stack_create(const pconv_handle* const* layers,
   if (e == cudaSuccess) e = cudaMemset(s->status_dev, 0, pconv::kStatusBlockBytes);
   if (e == cudaSuccess) e = cudaMallocHost(&s->status_host, sizeof(int));
   if (e == cudaSuccess) *s->status_host = 0;
-  if (e == cudaSuccess && !build_chains(s)) e = cudaErrorMemoryAllocation;
+  if (e == cudaSuccess && (!build_chains(s) || !build_rows(s))) e = cudaErrorMemoryAllocation;
   if (e != cudaSuccess) {
     cudaGetLastError();
     pconv_stack_free(s);
@@ -543,12 +646,10 @@ extern "C" pconv_status pconv_stack_launches(const pconv_stack* s, int* launches
     ++n;
     for (int k = i; k < last; ++k) {
       const pconv::DeviceLayer& L = s->layers[k]->d;
-      const unsigned sel_bits = PCONV_KERNEL_SIMPLE | PCONV_KERNEL_TILED | PCONV_KERNEL_GENERIC_TAPS | PCONV_KERNEL_TENSOR;
-      const bool tensor = (s->flags & PCONV_KERNEL_TENSOR) ||
-                          (!(s->flags & sel_bits) && pconv::tensor_preferred(L, s->n, ch, cw));
-      const bool fuse = s->pool[k] && !(s->flags & PCONV_KERNEL_SIMPLE) && !tensor &&
-                        pconv::tiled_supported(L, s->n, ch, cw);
+      const bool fuse = s->pool[k] && fuses_pool(s, k, ch, cw);
       if (!chain && s->pool[k] && !fuse) ++n;      // a max-pool kernel of its own
+      // position rows that the layer before does not write take a launch
+      if ((*s->rows)[k] && (k == 0 || (*s->path)[k - 1] == pconv::kNotDense)) ++n;
       ch = (ch - 1) / L.stride + 1;
       cw = (cw - 1) / L.stride + 1;
       if (s->pool[k]) {
@@ -593,19 +694,37 @@ extern "C" pconv_status pconv_stack_forward(pconv_stack* s, const void* x, void*
       continue;
     }
     const pconv::DeviceLayer& L = s->layers[i]->d;
-    // a pool that follows the layer is fused into the layer's epilogue when a tiled kernel runs it
-    // (not when the layer takes the dense tensor-core kernel, which has no pooled epilogue: the
-    // plain max-pool kernel follows it)
-    const unsigned sel_bits = PCONV_KERNEL_SIMPLE | PCONV_KERNEL_TILED | PCONV_KERNEL_GENERIC_TAPS | PCONV_KERNEL_TENSOR;
-    const bool tensor = (s->flags & PCONV_KERNEL_TENSOR) ||
-                        (!(s->flags & sel_bits) && pconv::tensor_preferred(L, s->n, ch, cw));
-    const bool fuse = s->pool[i] && !(s->flags & PCONV_KERNEL_SIMPLE) && !tensor &&
-                      pconv::tiled_supported(L, s->n, ch, cw);
+    const bool fuse = s->pool[i] && fuses_pool(s, i, ch, cw);
     const bool last_op = (i == s->n_layers - 1) && (!s->pool[i] || fuse);
     void* dst = last_op ? y : s->act[which];
-    pconv_status st = forward_impl(s->layers[i], cur, s->bias[i], dst, s->n, ch, cw,
-                                   s->flags | (fuse ? PCONV_POOL2X2 : 0u), s->ws, s->ws_bytes, stream,
-                                   s->status_dev);
+    pconv_status st = PCONV_OK;
+    if ((*s->path)[i] != pconv::kNotDense) {
+      // position rows in (written by the layer before where it is a dense one too, else staged here) or
+      // NCHW; and position rows out where the next layer takes them
+      void* rows = (*s->rows)[i];
+      pconv::DeviceLayer D = L;
+      D.err = s->status_dev;
+      cudaError_t e = cudaSuccess;
+      if (rows && cur != rows) e = pconv::launch_stage(D, cur, rows, s->n, ch, cw, fuse, (cudaStream_t)stream);
+      pconv::DenseNext next;
+      const bool to_rows = i + 1 < s->n_layers && (*s->rows)[i + 1];
+      if (to_rows) {
+        next = {L.c_out, s->layers[i + 1]->d.stride, s->pool[i + 1] != 0};
+        dst = (*s->rows)[i + 1];
+      }
+      const bool repro = (s->flags & PCONV_REPRODUCIBLE) != 0;
+      if (e == cudaSuccess)
+        e = pconv::launch_dense(D, rows ? rows : cur, s->bias[i], dst, s->n, ch, cw, (s->flags & PCONV_RELU) != 0, fuse, rows,
+                                to_rows ? &next : nullptr, repro ? nullptr : s->ws, repro ? 0 : s->ws_bytes,
+                                (cudaStream_t)stream);
+      if (e != cudaSuccess) {
+        cudaGetLastError();
+        return PCONV_ERR_CUDA;
+      }
+    } else {
+      st = forward_impl(s->layers[i], cur, s->bias[i], dst, s->n, ch, cw, s->flags | (fuse ? PCONV_POOL2X2 : 0u), s->ws,
+                        s->ws_bytes, nullptr, 0, stream, s->status_dev);
+    }
     if (st != PCONV_OK) return st;
     ch = (ch - 1) / L.stride + 1;
     cw = (cw - 1) / L.stride + 1;

@@ -2,6 +2,7 @@
 // extraction"), filter grouping balanced by surviving-kernel count and same-pattern ordering
 // inside a block ("filter kernel reorder"), and emission of the compressed value / code streams.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <memory>
@@ -100,30 +101,36 @@ extern "C" pconv_status pconv_pack(const float* w, int c_out, int c_in, const ui
     std::vector<std::vector<KernelRec>> per_filter(c_out);
     long long n_kept = 0;
     long long per_pattern[PCONV_MAX_PATTERNS] = {0};
+    signed char first_pattern[512];        // by support: the lowest pattern id that contains it, or -1
+    for (int m = 0; m < 512; ++m) {
+      first_pattern[m] = -1;
+      for (int p = n_patterns - 1; p >= 0; --p)
+        if ((m & ~(int)patterns[p]) == 0) first_pattern[m] = (signed char)p;
+    }
     for (int o = 0; o < c_out; ++o) {
       for (int c = 0; c < c_in; ++c) {
         const float* k = w + ((size_t)o * c_in + c) * 9;
-        unsigned support = 0;
+        uint32_t bits[9];
+        std::memcpy(bits, k, sizeof(bits));
+        if (!((bits[0] | bits[1] | bits[2] | bits[3] | bits[4] | bits[5] | bits[6] | bits[7] | bits[8]) & 0x7FFFFFFFu))
+          continue;                                      // pruned: most kernels are
+        unsigned support = 0, odd = 0;                   // non-zero taps; taps that are not finite
         for (int t = 0; t < 9; ++t) {
-          if (!std::isfinite(k[t])) {
-            if (bad_o) *bad_o = o;
-            if (bad_c) *bad_c = c;
-            return PCONV_ERR_RANGE;
-          }
-          if (k[t] != 0.0f) support |= 1u << t;
+          const uint32_t m = bits[t] & 0x7FFFFFFFu;
+          support |= (unsigned)(m != 0) << t;
+          odd |= (unsigned)(m >= 0x7F800000u);
         }
-        if (!support) continue;
+        if (odd) {
+          if (bad_o) *bad_o = o;
+          if (bad_c) *bad_c = c;
+          return PCONV_ERR_RANGE;
+        }
         if ((flags & PCONV_STRICT4) && popcount9(support) != 4) {
           if (bad_o) *bad_o = o;
           if (bad_c) *bad_c = c;
           return PCONV_ERR_KERNEL_NOT_IN_SET;
         }
-        int pid = -1;
-        for (int p = 0; p < n_patterns; ++p)
-          if ((support & ~(unsigned)patterns[p]) == 0) {
-            pid = p;
-            break;
-          }
+        const int pid = first_pattern[support];
         if (pid < 0) {
           if (bad_o) *bad_o = o;
           if (bad_c) *bad_c = c;
@@ -206,7 +213,11 @@ extern "C" pconv_status pconv_pack(const float* w, int c_out, int c_in, const ui
     std::vector<uint16_t> wv16;
     long long max_gk = 0, min_gk = -1;
     struct Item { int c, canon_or_pid, slot; const KernelRec* r; };
-    std::vector<Item> items;
+    std::vector<Item> items, sorted;
+    std::vector<uint16_t> rec;
+    codes_s.reserve((size_t)n_kept * 3 + (size_t)n_groups * n_chunks * 64);
+    codes_g.reserve((size_t)n_kept * 2 + (size_t)n_groups * n_chunks * 48);
+    (storage == PCONV_F16 ? wv16.reserve(4 * n_kept + 8) : wv32.reserve(4 * n_kept + 8));
     std::vector<size_t> cursor(c_out, 0);
     for (int g = 0; g < n_groups; ++g) {
       long long gk = 0;
@@ -229,12 +240,14 @@ extern "C" pconv_status pconv_pack(const float* w, int c_out, int c_in, const ui
             ++cur;
           }
         }
-        // channel-major; inside a channel, same-pattern kernels adjacent, then by slot
-        std::stable_sort(items.begin(), items.end(), [](const Item& a, const Item& b) {
-          if (a.c != b.c) return a.c < b.c;
-          if (a.canon_or_pid != b.canon_or_pid) return a.canon_or_pid < b.canon_or_pid;
-          return a.slot < b.slot;
-        });
+        // channel-major; inside a channel, same-pattern kernels adjacent, then by slot: a counting sort
+        // over (channel, pattern), which keeps the slots' order
+        int start[kChunk * PCONV_MAX_PATTERNS + 1] = {0};
+        for (const Item& it : items) ++start[(it.c - c0) * PCONV_MAX_PATTERNS + it.canon_or_pid + 1];
+        for (int i = 0; i < kChunk * PCONV_MAX_PATTERNS; ++i) start[i + 1] += start[i];
+        sorted.resize(items.size());
+        for (const Item& it : items) sorted[start[(it.c - c0) * PCONV_MAX_PATTERNS + it.canon_or_pid]++] = it;
+        items.swap(sorted);
         BlockDesc& bd = blocks[(size_t)g * n_chunks + k];
         std::memset(&bd, 0, sizeof(bd));
         bd.w_off = (uint32_t)((storage == PCONV_F16 ? wv16.size() : wv32.size()) / 4);
@@ -249,7 +262,7 @@ extern "C" pconv_status pconv_pack(const float* w, int c_out, int c_in, const ui
         // record) that can name every mask's body.
         const bool wide = !h->canonical;
         const int per_record = wide ? kWideCodesPerRecord : kCodesPerRecord;
-        std::vector<uint16_t> rec;
+        rec.clear();
         auto close_record = [&](uint16_t terminator) {
           rec.push_back(terminator);
           while ((int)rec.size() < per_record) rec.push_back((uint16_t)(wide ? kWideEnd : kCodeEnd));
@@ -299,34 +312,6 @@ extern "C" pconv_status pconv_pack(const float* w, int c_out, int c_in, const ui
     for (int i = 0; i < 32; ++i) { codes_s.push_back(0); codes_s.push_back(0); codes_g.push_back(0); }
     for (int i = 0; i < 8; ++i) { wv32.push_back(0.f); wv16.push_back(0); }
 
-    // ---- zero-inserted dense weights for the tensor-core path (fp16 storage, stride 1) ----------
-    // Filters in original order, tiles of 64 (layers of up to 64 filters) or 128; channels padded to
-    // a multiple of 16 with zeros.  Left out for layers whose dense form would exceed 64 MB.
-    std::vector<uint16_t> wdense;
-    int dense_nt = 0;
-    if (storage == PCONV_F16 && stride == 1) {
-      const int nt = c_out <= 64 ? 64 : 128;
-      const size_t n_tiles = (size_t)(c_out + nt - 1) / nt, k_steps = (size_t)(c_in + 15) / 16;
-      const size_t halves = n_tiles * k_steps * 9 * nt * 16;
-      if (halves * 2 <= ((size_t)64 << 20)) {
-        dense_nt = nt;
-        wdense.assign(halves, 0);
-        for (int o = 0; o < c_out; ++o) {
-          const size_t tile = (size_t)o / nt, on = (size_t)o % nt;
-          for (const KernelRec& r : per_filter[o]) {
-            const size_t ks = (size_t)r.c / 16, kc = (size_t)r.c % 16;
-            int s = 0;
-            for (int t = 0; t < 9; ++t) {
-              if (!(patterns[r.pid] >> t & 1)) continue;
-              const size_t idx = ((((tile * k_steps + ks) * 9 + t) * 2 + kc / 8) * (nt / 8) + on / 8) * 64 +
-                                 (on % 8) * 8 + kc % 8;
-              wdense[idx] = r.hv[s++];
-            }
-          }
-        }
-      }
-    }
-
     // ---- one device allocation, sub-buffers 256-byte aligned ------------------------------------
     struct Part { const void* src; size_t bytes; size_t off; };
     auto align256 = [](size_t v) { return (v + 255) & ~(size_t)255; };
@@ -349,7 +334,17 @@ extern "C" pconv_status pconv_pack(const float* w, int c_out, int c_in, const ui
     const int i_pm = add(perm.data(), perm.size() * 4);
     const std::vector<unsigned char> zero_block(kStatusBlockBytes, 0);
     const int i_er = add(zero_block.data(), zero_block.size());
-    const int i_wd = dense_nt ? add(wdense.data(), wdense.size() * 2) : -1;
+    // zero-inserted weights of the dense tensor-core path: built on the device from the lists above
+    DeviceLayer& d = h->d;
+    d.c_out = c_out;
+    d.c_in = c_in;
+    d.stride = stride;
+    d.storage = storage;
+    d.dense_rows = (c_out + 15) / 16 * 16;
+    for (int p = 0; p < n_patterns; ++p)
+      if (per_pattern[p]) d.tap_mask |= patterns[p];
+    const bool dense = d.tap_mask && dense_weight_bytes(d) <= kMaxDenseBytes;
+    const int i_wd = dense ? add(nullptr, dense_weight_bytes(d)) : -1;
 
     char* dev = nullptr;
     if (cudaMalloc((void**)&dev, total) != cudaSuccess) {
@@ -358,9 +353,23 @@ extern "C" pconv_status pconv_pack(const float* w, int c_out, int c_in, const ui
     }
     cudaError_t e = cudaSuccess;
     for (int i = 0; i < np && e == cudaSuccess; ++i)
-      if (parts[i].bytes)
+      if (parts[i].bytes && parts[i].src)
         e = cudaMemcpyAsync(dev + parts[i].off, parts[i].src, parts[i].bytes,
                             cudaMemcpyHostToDevice, stream);
+    d.row_ptr = (const int*)(dev + parts[i_rp].off);
+    d.csr_idx = (const uint32_t*)(dev + parts[i_ci].off);
+    d.csr_val = (const float*)(dev + parts[i_cv].off);
+    d.blocks = (const BlockDesc*)(dev + parts[i_bl].off);
+    d.wvals = dev + parts[i_wv].off;
+    d.codes_s = (const uint8_t*)(dev + parts[i_cs].off);
+    d.wide_codes = h->canonical ? 0 : 1;
+    d.codes_g = (const uint8_t*)(dev + parts[i_cg].off);
+    d.perm = (const int*)(dev + parts[i_pm].off);
+    d.err = (int*)(dev + parts[i_er].off);
+    d.wdense = i_wd >= 0 ? dev + parts[i_wd].off : nullptr;
+    static std::atomic<long long> layer_ids{0};
+    d.id = ++layer_ids;
+    if (e == cudaSuccess && d.wdense) e = dense_build_weights(d, stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
     if (e != cudaSuccess) {
       cudaGetLastError();
@@ -373,23 +382,6 @@ extern "C" pconv_status pconv_pack(const float* w, int c_out, int c_in, const ui
     h->wvals_bytes = parts[i_wv].bytes;
     h->codes_s_bytes = parts[i_cs].bytes;
     h->codes_g_bytes = parts[i_cg].bytes;
-    DeviceLayer& d = h->d;
-    d.row_ptr = (const int*)(dev + parts[i_rp].off);
-    d.csr_idx = (const uint32_t*)(dev + parts[i_ci].off);
-    d.csr_val = (const float*)(dev + parts[i_cv].off);
-    d.blocks = (const BlockDesc*)(dev + parts[i_bl].off);
-    d.wvals = dev + parts[i_wv].off;
-    d.codes_s = (const uint8_t*)(dev + parts[i_cs].off);
-    d.wide_codes = h->canonical ? 0 : 1;
-    d.codes_g = (const uint8_t*)(dev + parts[i_cg].off);
-    d.perm = (const int*)(dev + parts[i_pm].off);
-    d.err = (int*)(dev + parts[i_er].off);
-    d.wdense = i_wd >= 0 ? dev + parts[i_wd].off : nullptr;
-    d.dense_nt = dense_nt;
-    d.c_out = c_out;
-    d.c_in = c_in;
-    d.stride = stride;
-    d.storage = storage;
     d.n_groups = n_groups;
     d.n_chunks = n_chunks;
     d.n_kept = n_kept;

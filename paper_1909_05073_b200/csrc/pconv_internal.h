@@ -88,11 +88,13 @@ struct DeviceLayer {         // device pointers of one packed layer (passed to k
   int c_out, c_in, stride, storage, n_groups, n_chunks;
   int wide_codes;            // 0 = narrow codes (canonical set), 1 = wide codes
   long long n_kept;          // surviving kernels of the layer
-  // zero-inserted dense fp16 weights for the tensor-core path (fp16 storage, stride 1; else null):
-  // per (filter tile of dense_nt, 16-channel step) nine [dense_nt x 16] matrices in the K-major
-  // core-matrix order of tcgen05 shared-memory descriptors: [tap][k half][filter / 8][filter % 8][k % 8]
+  // zero-inserted weights for the dense tensor-core path (null if the layer has none), written by
+  // dense_build_weights: per (16-channel step, stored tap, 8 channels, piece) one 16-byte row of 8
+  // channels per filter; fp16 storage has one piece (the values), fp32 three (bf16, summing up exactly)
   const void* wdense;
-  int dense_nt;
+  int dense_rows;            // filters rounded up to 16
+  int tap_mask;              // union of the layer's pattern masks: the taps that are stored
+  long long id;              // unique per packed layer of the process (from 1)
 };
 
 // Status block: one status word, one pad word, kTraceWords 64-bit trace words (written only by
@@ -130,11 +132,27 @@ cudaError_t launch_simple(const DeviceLayer& L, const void* x, const float* bias
 cudaError_t launch_tiled(const DeviceLayer& L, const void* x, const float* bias, void* y, int n,
                          int h, int w, bool relu, bool pool, bool reproducible, bool generic_taps,
                          int rmode, bool allow_cluster, void* ws, size_t ws_bytes, cudaStream_t stream);
-cudaError_t launch_tensor(const DeviceLayer& L, const void* x, const float* bias, void* y, int n,
-                          int h, int w, bool relu, void* ws, size_t ws_bytes, cudaStream_t stream);
-size_t tensor_workspace_bytes(const DeviceLayer& L, int n, int h, int w);
-bool tensor_supported(const DeviceLayer& L, int n, int h, int w);
-bool tensor_preferred(const DeviceLayer& L, int n, int h, int w);
+// dense tensor-core path (kernels_dense.cu)
+constexpr size_t kMaxDenseBytes = (size_t)256 << 20;   // layers whose dense weights would exceed this have none
+constexpr size_t kMaxSplitBytes = (size_t)24 << 20;    // workspace a split may ask for
+size_t dense_weight_bytes(const DeviceLayer& L);
+cudaError_t dense_build_weights(const DeviceLayer& L, cudaStream_t stream);
+bool dense_supported(const DeviceLayer& L, int n, int h, int w, bool pool);
+enum RowsFrom { kNoRows, kRowsStaged, kRowsGiven };    // position rows: no room, to be staged, already there
+enum DensePath { kNotDense, kFromNchw, kFromRows };
+DensePath dense_path(const DeviceLayer& L, int n, int h, int w, bool pool, RowsFrom rows, size_t ws_bytes);
+size_t dense_workspace_bytes(const DeviceLayer& L, int n, int h, int w, size_t most);
+// Activations in the dense kernel's own layout ("position rows", see kernels_dense.cu): the size of a
+// layer's input in it (0 = the shape has no such form), and the kernel that makes it from NCHW.
+size_t dense_rows_bytes(const DeviceLayer& L, int n, int h, int w, bool pool);
+cudaError_t launch_stage(const DeviceLayer& L, const void* x, void* rows, int n, int h, int w, bool pool,
+                         cudaStream_t stream);
+struct DenseNext { int c_in, stride; bool pool; };   // the layer that reads the result as position rows
+// rows_in: x is position rows, not NCHW; next: y becomes the next layer's position rows (whose padding
+// must be zero already).
+cudaError_t launch_dense(const DeviceLayer& L, const void* x, const float* bias, void* y, int n, int h, int w,
+                         bool relu, bool pool, bool rows_in, const DenseNext* next, void* ws, size_t ws_bytes,
+                         cudaStream_t stream);
 // rmode: what the caller pinned for the tiled kernel: output rows per lane (4, 8, or 0 = the planner
 // chooses) | kPinBulk (fp32 chunks fetched by bulk copies into a raw ring)
 constexpr int kPinRowsMask = 0xff;
@@ -144,7 +162,8 @@ bool tiled_supported(const DeviceLayer& L, int n, int h, int w);
 bool tiled_plan(const DeviceLayer& L, int n, int h, int w, bool generic_taps, bool with_workspace,
                 int rmode, pconv_plan_t* out);
 #ifdef PCONV_DEV
-cudaError_t dev_set_withhold(int chunk, unsigned spin_limit);   // see pconv_dev.h
+cudaError_t dev_set_withhold(int chunk, unsigned spin_limit);     // see pconv_dev.h
+cudaError_t dense_set_withhold(int step, unsigned spin_limit);
 #endif
 // chains: several consecutive layers of a stack in one persistent launch (kernels_tiled.cu)
 bool chain_layer_ok(const DeviceLayer& L, int n, int h, int w, bool pool, long long* ctas);
