@@ -43,6 +43,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -63,6 +64,7 @@ constexpr int kBiasOff = 512;
 constexpr uint32_t kSpinLimit = 1u << 20;
 constexpr uint32_t kWaitHintNs = 200;
 constexpr int kSmemLimit = 227 * 1024;
+constexpr int kTables = 5;                // load tables of the NCHW producers: segments s - 1 .. s + 3
 
 // P8: the activations come in position rows (see stage_kernel) that bulk copies move; otherwise the
 // producer warps convert them from NCHW.
@@ -90,6 +92,7 @@ struct DGeo {
   int vec, n_vec, vec_rows, vec_cols, row_planes;   // loads: pixels of one, loads of a channel, their grid
   int tiles, pool, mpos;             // MMA tiles of an item, fused pool, positions of an item
   int nt, n_ft, form3;               // filters of a tile (multiple of 16), filter tiles; fp32: see kernel
+  int out_col, out_stride;           // fp32: columns the finished sums go to (0: over the main sums), tiles' distance
   int tile_cols, n_buf;              // Tensor Memory columns of a tile; accumulator sets (fp16)
   int rows;                          // filter rows in the weight stream (c_out rounded up to 16)
   int n_taps, tps, slots;            // taps stored; taps of a ring slot; slots of a channel step
@@ -97,6 +100,7 @@ struct DGeo {
   int a_stages, b_slots, a_off, b_off, a_bytes, b_bytes;
   int relu;
   int n_tiles, grid;                 // (positions, filters) tiles, CTAs
+  int cluster;                       // the CTAs of a tile are a thread-block cluster and exchange their sums directly
   int share, share_more, parts;      // a CTA's tiles or steps (the first share_more: one more); equal parts of a tile
   int in_plane_len, in_lead;         // P8 source: positions of a plane, positions before the batch's first
   int out_p8, out_pitch, out_cell_rows, out_sy, out_sx, out_plane_len, out_lead;   // P8 result: the next layer's rows
@@ -247,6 +251,12 @@ __device__ __forceinline__ void tmem_ld16(uint32_t (&v)[16], uint32_t taddr) {
                  "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
                : "r"(taddr));
 }
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const float* v) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "f"(v[0]), "f"(v[1]),
+               "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+               : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void red_add_v4(float* p, float a, float b, float c, float d) {
   asm volatile("red.global.v4.f32.add [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
@@ -261,6 +271,10 @@ __device__ __forceinline__ int take_ticket(int* p) {
 // anywhere, but at least kMinSteps from one.  A CTA's share is a few segments, each inside one tile.
 constexpr int kMinSteps = 2;
 __host__ __device__ inline int share_begin(const DGeo& g, int cta) {
+  if (g.cluster) {
+    const int t = cta / g.parts;
+    return t * g.k_steps + (cta - t * g.parts) * g.k_steps / g.parts;
+  }
   const int x = cta * g.share + (cta < g.share_more ? cta : g.share_more);   // (tiles, or steps if split)
   if (!g.split) return x * g.k_steps;
   if (g.parts) return x;
@@ -475,6 +489,58 @@ __device__ __forceinline__ void store_rows(void* __restrict__ y, const DGeo& g, 
   }
 }
 
+// Bias, ReLU and store of eight finished columns (filters f0 + col ..) of this lane's position.
+template <bool HALF>
+__device__ __forceinline__ void finish_columns(const DGeo& g, void* __restrict__ y, float (&v)[8], const float* bias_s,
+                                               long long dst, int f0, int col, int n_f, size_t plane, bool pool,
+                                               bool pairs, int lane) {
+  typedef typename std::conditional<HALF, __half, float>::type T;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    v[i] += bias_s[(col + i) & 127];
+    if (g.relu) v[i] = fmaxf(v[i], 0.f);
+  }
+  if (g.out_p8) {
+    // (the last filter tile may reach past the layer's filters, and so past the next layer's groups)
+    if (f0 + col < g.rows) store_rows<HALF>(y, g, v, dst, (f0 + col) >> 3, pool, lane);
+  } else {
+    store_chunk(reinterpret_cast<T*>(y), v, dst, col, n_f, plane, pool, pairs, lane);
+  }
+}
+// Where a lane's position goes: element offset at filter f0, or plane and position; -1: nowhere.
+__device__ __forceinline__ long long lane_dest(const DGeo& g, int p, int f0, size_t plane) {
+  const long long d = position_dest(g, p);
+  return g.out_p8 || d < 0 ? d : d + (long long)f0 * (long long)plane;
+}
+// With a fused pool two tiles are the two rows of the same positions, the two lanes of a pair the two
+// columns.
+__device__ __forceinline__ void pool_columns(float (&v)[8], const float (&v2)[8]) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    v[i] = fmaxf(v[i], v2[i]);
+    v[i] = fmaxf(v[i], __shfl_xor_sync(0xffffffffu, v[i], 1));
+  }
+}
+
+// All threads of a cluster's CTAs meet; writes before it are seen after it.
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ float4 ld_cluster(uint32_t addr, uint32_t rank) {
+  float4 v;
+  asm volatile(
+      "{\n\t.reg .b32 a;\n\tmapa.shared::cluster.u32 a, %4, %5;\n\t"
+      "ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [a];\n\t}"
+      : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+      : "r"(addr), "r"(rank)
+      : "memory");
+  return v;
+}
+// Sums of a warp's columns for the other CTAs of the cluster: [column / 4][warp][lane][4] fp32.
+__device__ __forceinline__ uint32_t exchange_addr(uint32_t base, int c4, int warp, int lane) {
+  return base + (uint32_t)((c4 * 8 + warp) * 32 + lane) * 16u;
+}
+
 // Warp roles share these shared-memory addresses.
 struct Bars {
   uint32_t af, ae, bf, be, cf, ce;    // activations, weights, accumulators: full / empty
@@ -499,6 +565,8 @@ __device__ __forceinline__ void mma_role(const DeviceLayer& L, const DGeo& g, ui
     const uint32_t id0 = (1u << 4) | (HALF ? 0u : (1u << 7) | (1u << 10)) | ((128u >> 4) << 24);
     const uint32_t nt = (uint32_t)g.nt;
     const uint32_t id1 = id0 | ((nt >> 3) << 17), id2 = id0 | ((2 * nt >> 3) << 17), id3 = id0 | ((3 * nt >> 3) << 17);
+    // (in a cluster a shared-memory address carries the CTA's rank above its 18 bits; descriptors do not)
+    const uint32_t sdesc = sbase & 0x3FFFFu;
     const u64 a_d0 = smem_desc(0u, (uint32_t)g.q_tot * 16u, 128u);
     const u64 b_d0 = smem_desc(0u, (uint32_t)(C::kPieces * g.nt) * 16u, 128u);
     const uint32_t slab = 2u * (uint32_t)g.q_tot;        // 16-byte rows of one piece of a stage
@@ -518,7 +586,7 @@ __device__ __forceinline__ void mma_role(const DeviceLayer& L, const DGeo& g, ui
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     };
     auto slot_desc = [&](int s) -> u64 {
-      return b_d0 + ((sbase + (uint32_t)g.b_off + (uint32_t)s * (uint32_t)g.b_bytes) >> 4);
+      return b_d0 + ((sdesc + (uint32_t)g.b_off + (uint32_t)s * (uint32_t)g.b_bytes) >> 4);
     };
     Item it;
     for (int seg = 0; get_item(g, share, seg, &it); ++seg) {
@@ -528,7 +596,7 @@ __device__ __forceinline__ void mma_role(const DeviceLayer& L, const DGeo& g, ui
         const uint32_t d0 = tmem + buf * 256u;
         for (int ks = it.k0; ks < it.k1; ++ks) {
           wait(bar.af + 8 * sa, pa, 2, 2);
-          const u64 a_st = a_d0 + ((sbase + (uint32_t)g.a_off + (uint32_t)sa * (uint32_t)g.a_bytes) >> 4);
+          const u64 a_st = a_d0 + ((sdesc + (uint32_t)g.a_off + (uint32_t)sa * (uint32_t)g.a_bytes) >> 4);
 #pragma unroll
           for (int t = 0; t < 9; t += 3) {                 // three taps to a slot
             if (t >= g.n_taps) break;
@@ -558,7 +626,7 @@ __device__ __forceinline__ void mma_role(const DeviceLayer& L, const DGeo& g, ui
           const bool first = ks == it.k0;
           if (first) wait(bar.ce, (sc & 1u) ^ 1u, 3, 1);
           wait(bar.af + 8 * sa, pa, 2, 2);
-          const u64 a_st = a_d0 + ((sbase + (uint32_t)g.a_off + (uint32_t)sa * (uint32_t)g.a_bytes) >> 4);
+          const u64 a_st = a_d0 + ((sdesc + (uint32_t)g.a_off + (uint32_t)sa * (uint32_t)g.a_bytes) >> 4);
           auto cross = [&](int j, int t, u64 b_t) {
             const u64 a1 = a_st + (uint32_t)g.tap_off[j][t], a2 = a1 + slab, a3 = a2 + slab;
             const uint32_t dc = tmem + (uint32_t)(j * g.tile_cols) + nt;
@@ -739,7 +807,7 @@ dense_kernel(const DeviceLayer L, const __grid_constant__ DGeo g, const void* __
   const uint32_t bar_cf = bar_be + 8 * kMaxB, bar_ce = bar_cf + 16;     // accumulators full / empty
   volatile uint32_t* tmem_s = reinterpret_cast<volatile uint32_t*>(smem + 16 * (kMaxA + kMaxB) + 32);
   float* bias_s = reinterpret_cast<float*>(smem + kBiasOff);            // [128]
-  Load* tab_s = reinterpret_cast<Load*>(smem + kHeader);                // [4][n_vec]
+  Load* tab_s = reinterpret_cast<Load*>(smem + kHeader);                // [kTables][n_vec]
 
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (tid == 0) T_STAMP(10);
@@ -802,16 +870,15 @@ dense_kernel(const DeviceLayer L, const __grid_constant__ DGeo g, const void* __
     const uint32_t half_b = (uint32_t)g.q_tot * 16u, slab = 2u * half_b;
     const int withhold = D_WITHHOLD_STEP;     // (development build: a step whose first warp never reports)
     T_DECL;
-    // The loads of an item: worked out two items ahead of the stores, because the loads run up to two
-    // batches ahead of them and an item may be as short as one batch.
+    // The loads of a segment: worked out three segments ahead of the stores.  A segment may be as short as
+    // one batch, and two batches beyond the one to be stored next are loaded before its segment begins.
     auto fill_table = [&](int seg) {
       Item it;
       if (!get_item(g, share, seg, &it)) return;
-      Load* tab = tab_s + (seg & 3) * g.n_vec;
+      Load* tab = tab_s + (seg % kTables) * g.n_vec;
       for (int u = pt; u < g.n_vec; u += C::kProdThreads) tab[u] = decode_load(g, it.m0, u);
     };
-    fill_table(0);
-    fill_table(1);
+    for (int i = 0; i < 3; ++i) fill_table(i);
     bool ok = role_all<1, C::kProdThreads>(true);
     // the previous kernel of the stream has finished before x is read
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -830,7 +897,7 @@ dense_kernel(const DeviceLayer L, const __grid_constant__ DGeo g, const void* __
       if (!get_item(g, share, l_seg, &it)) return;
       l_ks = it.k0;
       l_k1 = it.k1;
-      l_tab = tab_s + (l_seg & 3) * g.n_vec;
+      l_tab = tab_s + (l_seg % kTables) * g.n_vec;
     };
     open_item();
     auto load_batch = [&](Set& r) {
@@ -869,7 +936,7 @@ dense_kernel(const DeviceLayer L, const __grid_constant__ DGeo g, const void* __
         if (!get_item(g, share, s_seg, &it)) return false;
         s_ks = s_k0 = it.k0;
         s_k1 = it.k1;
-        fill_table(s_seg + 2);
+        fill_table(s_seg + 3);
         ok = role_all<1, C::kProdThreads>(ok);
         if (!ok) return false;
       }
@@ -923,8 +990,6 @@ dense_kernel(const DeviceLayer L, const __grid_constant__ DGeo g, const void* __
     }
   } else {
     // ======================================= epilogue =========================================
-    typedef typename std::conditional<HALF, __half, float>::type T;
-    T* y = reinterpret_cast<T*>(yv);
     // fp32 keeps a warp's columns of all tiles in registers: kSums of one tile or half as many of each of two
     constexpr int kSums = HALF ? 8 : (P8 ? 128 : 64), kHalf = kSums / 2;
     const int q = warp & 3, grp = warp >> 2;             // lane quadrant, column group
@@ -987,8 +1052,19 @@ dense_kernel(const DeviceLayer L, const __grid_constant__ DGeo g, const void* __
           take(g.nt);
           if (g.form3) take(2 * g.nt);
         }
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        warp_arrive(bar_ce, lane);
+        // The sums go back to Tensor Memory, which can be addressed at run time: what follows is then one short
+        // loop over columns.  (Unrolled over registers it was 38 KB of code run once per tile, and fetching
+        // the instructions took 10 us.)  Where all columns are in use they replace the main sums.
+#pragma unroll
+        for (int k = 0; k < kSums; k += 8) {
+          const int j = g.tiles == 2 ? k / kHalf : 0, c = g.tiles == 2 ? k % kHalf : k;
+          if (c < n_col) tmem_st8(lane_addr + (uint32_t)(g.out_col + j * g.out_stride + c), sum + k);
+        }
+        tmem_st_wait();
+        if (g.out_col) {
+          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+          warp_arrive(bar_ce, lane);
+        }
       }
       if (!waited) {   // the previous kernel of the stream has finished before y or the workspace is written
         asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -996,34 +1072,40 @@ dense_kernel(const DeviceLayer L, const __grid_constant__ DGeo g, const void* __
       }
       ok = role_all<2, 32 * C::kEpiWarps>(ok);             // the bias is staged
       if (!ok) break;
+      const uint32_t res = lane_addr + (HALF ? buf * 256u : (uint32_t)g.out_col);     // this warp's columns of tile 0
+      const uint32_t res_stride = (uint32_t)(HALF ? g.tile_cols : g.out_stride);
+      if (g.cluster) {   // this CTA's only segment: hand the sums over (the rings are free: all MMAs are done)
+        for (int j = 0; j < g.tiles; ++j)
+#pragma unroll 1
+          for (int c = 0; c < n_col; c += 8) {
+            uint32_t v[8];
+            tmem_ld8(v, res + (uint32_t)j * res_stride + (uint32_t)c);
+            tmem_ld_wait();
+            const int c4 = (j * n_col + c) / 4;
+            const uint32_t lo[4] = {v[0], v[1], v[2], v[3]}, hi[4] = {v[4], v[5], v[6], v[7]};
+            sts128(exchange_addr(sbase + (uint32_t)g.a_off, c4, warp, lane), lo);
+            sts128(exchange_addr(sbase + (uint32_t)g.a_off, c4 + 1, warp, lane), hi);
+          }
+        continue;
+      }
       // Parts of the channel range: add this part's sums to the tile's in the workspace
       // ([tile][column / 4][position][4]: 16 bytes a lane), take a ticket for this warp's share; the
       // warp that draws the last one reads the sums back (zeroing them) and finishes.
-      float* wsw = nullptr;
       bool finish = true;
-      const bool part = it.k1 - it.k0 < g.k_steps;
-      if (part) {
+      if (it.k1 - it.k0 < g.k_steps) {
         int slot, parts;
         tile_owners(g, it.tile, &slot, &parts);
-        wsw = ws + ((size_t)slot * g.tiles * (g.nt / 4) + (size_t)(col0 / 4)) * 512 + (size_t)(32 * q + lane) * 4;
-        if constexpr (HALF) {
-          for (int j = 0; j < g.tiles; ++j)
-            for (int c = 0; c < n_col; c += 8) {
-              uint32_t v[8];
-              tmem_ld8(v, lane_addr + buf * 256u + (uint32_t)(j * g.tile_cols + c));
-              tmem_ld_wait();
-              float* pw = wsw + ((size_t)j * (g.nt / 4) + c / 4) * 512;
-              red_add_v4(pw, __uint_as_float(v[0]), __uint_as_float(v[1]), __uint_as_float(v[2]), __uint_as_float(v[3]));
-              red_add_v4(pw + 512, __uint_as_float(v[4]), __uint_as_float(v[5]), __uint_as_float(v[6]),
-                         __uint_as_float(v[7]));
-            }
-        }
-        if (!HALF) {
-          float* pw = wsw;
-#pragma unroll
-          for (int k = 0; k < kSums; k += 4, pw += 512) {
-            if (k == kHalf && g.tiles == 2) pw = wsw + (size_t)(g.nt / 4) * 512;
-            if ((g.tiles == 2 ? k % kHalf : k) < n_col) red_add_v4(pw, sum[k], sum[k + 1], sum[k + 2], sum[k + 3]);
+        float* wsw = ws + ((size_t)slot * g.tiles * (g.nt / 4) + (size_t)(col0 / 4)) * 512 + (size_t)(32 * q + lane) * 4;
+        for (int j = 0; j < g.tiles; ++j) {
+          float* pw = wsw + (size_t)(j * (g.nt / 4)) * 512;
+#pragma unroll 1
+          for (int c = 0; c < n_col; c += 8, pw += 1024) {
+            uint32_t v[8];
+            tmem_ld8(v, res + (uint32_t)j * res_stride + (uint32_t)c);
+            tmem_ld_wait();
+            red_add_v4(pw, __uint_as_float(v[0]), __uint_as_float(v[1]), __uint_as_float(v[2]), __uint_as_float(v[3]));
+            red_add_v4(pw + 512, __uint_as_float(v[4]), __uint_as_float(v[5]), __uint_as_float(v[6]),
+                       __uint_as_float(v[7]));
           }
         }
         __syncwarp();
@@ -1034,125 +1116,52 @@ dense_kernel(const DeviceLayer L, const __grid_constant__ DGeo g, const void* __
           if (t == parts - 1) *ticket = 0;
         }
         finish = __shfl_sync(0xffffffffu, t, 0) == parts - 1;
-      }
-      const long long t_fin = T_NOW();
-      if (finish) {
-        // Up to 32 columns of tile j from c on: from the workspace (leaving zeros) or, for fp16, Tensor Memory.
-        // All loads are in flight together: one after the other they cost a trip to L2 each.
-        auto fetch = [&](int j, int c, float (&v)[32]) {
-          if (part) {
-            float4* p = reinterpret_cast<float4*>(wsw + ((size_t)j * (g.nt / 4) + c / 4) * 512);
+        for (int j = 0; finish && j < g.tiles; ++j)
+#pragma unroll 1
+          for (int c = 0; c < n_col; c += 32) {       // (eight loads in flight)
+            float4* pw = reinterpret_cast<float4*>(wsw + (size_t)(j * (g.nt / 4) + c / 4) * 512);
+            float v[32];
 #pragma unroll
             for (int i = 0; i < 8; ++i)
               if (c + 4 * i < n_col) {
-                const float4 a = __ldcg(p + 128 * i);
+                const float4 a = __ldcg(pw + 128 * i);
                 v[4 * i] = a.x; v[4 * i + 1] = a.y; v[4 * i + 2] = a.z; v[4 * i + 3] = a.w;
               }
 #pragma unroll
             for (int i = 0; i < 8; ++i)
-              if (c + 4 * i < n_col) p[128 * i] = make_float4(0.f, 0.f, 0.f, 0.f);
-          } else if (HALF) {
+              if (c + 4 * i < n_col) pw[128 * i] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-            for (int i = 0; i < 32; i += 16)
-              if (c + i < n_col) {
-                uint32_t r[16];
-                tmem_ld16(r, lane_addr + buf * 256u + (uint32_t)(j * g.tile_cols + c + i));
-#pragma unroll
-                for (int k = 0; k < 16; ++k) v[i + k] = __uint_as_float(r[k]);
-              }
+            for (int i = 0; i < 32; i += 8)
+              if (c + i < n_col) tmem_st8(res + (uint32_t)j * res_stride + (uint32_t)(c + i), v + i);
+            tmem_st_wait();
+          }
+      }
+      const long long t_fin = T_NOW();
+      if (finish) {
+        const int jstep = pool ? 2 : 1;
+        for (int j = 0, jj = 0; j < g.tiles; j += jstep, ++jj) {
+          const long long dst = lane_dest(g, it.m0 + 128 * jj + 32 * q + lane, it.f0, plane);
+#pragma unroll 1
+          for (int c = 0; c < n_col; c += 8) {
+            uint32_t r[8], r2[8];
+            tmem_ld8(r, res + (uint32_t)j * res_stride + (uint32_t)c);
+            if (pool) tmem_ld8(r2, res + (uint32_t)(j + 1) * res_stride + (uint32_t)c);
             tmem_ld_wait();
-          }
-        };
-        auto emit = [&](float (&v)[8], int c, long long dst) {
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            v[i] += bias_s[(col0 + c + i) & 127];
-            if (g.relu) v[i] = fmaxf(v[i], 0.f);
-          }
-          if (g.out_p8) {
-            // (the last filter tile may reach past the layer's filters, and so past the next layer's groups)
-            if (it.f0 + col0 + c < g.rows) store_rows<HALF>(yv, g, v, dst, (it.f0 + col0 + c) >> 3, pool, lane);
-            return;
-          }
-          // a warp stores its own columns only
-          store_chunk(y, v, dst, col0 + c, min(n_f, col0 + n_col), plane, pool, pairs, lane);
-        };
-        auto dest = [&](int jj) {
-          const long long d = position_dest(g, it.m0 + 128 * jj + 32 * q + lane);
-          if (g.out_p8) return d;
-          return d < 0 ? d : d + (long long)it.f0 * (long long)plane;
-        };
-        // with a fused pool two tiles are the two rows of the same positions, the two lanes of a pair
-        // the two columns
-        auto emit8 = [&](float (&v)[8], const float (&v2)[8], int c, long long dst) {
-          if (pool) {
+            float v[8], v2[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
-              v[i] = fmaxf(v[i], v2[i]);
-              v[i] = fmaxf(v[i], __shfl_xor_sync(0xffffffffu, v[i], 1));
+              v[i] = __uint_as_float(r[i]);
+              v2[i] = __uint_as_float(r2[i]);
             }
-          }
-          emit(v, c, dst);
-        };
-        if constexpr (!HALF) {
-          if (part) {
-            float* pw = wsw;
-#pragma unroll
-            for (int k = 0; k < kSums; k += 4, pw += 512) {
-              if (k == kHalf && g.tiles == 2) pw = wsw + (size_t)(g.nt / 4) * 512;
-              if ((g.tiles == 2 ? k % kHalf : k) < n_col) {
-                const float4 a = __ldcg(reinterpret_cast<const float4*>(pw));
-                sum[k] = a.x; sum[k + 1] = a.y; sum[k + 2] = a.z; sum[k + 3] = a.w;
-              }
-            }
-            pw = wsw;
-#pragma unroll
-            for (int k = 0; k < kSums; k += 4, pw += 512) {
-              if (k == kHalf && g.tiles == 2) pw = wsw + (size_t)(g.nt / 4) * 512;
-              if ((g.tiles == 2 ? k % kHalf : k) < n_col)
-                *reinterpret_cast<float4*>(pw) = make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-          }
-          long long dst = dest(0);
-#pragma unroll
-          for (int k = 0; k < kSums; k += 8) {
-            if (k == kHalf && g.tiles == 2) {
-              if (pool) break;
-              dst = dest(1);
-            }
-            const int c = g.tiles == 2 ? k % kHalf : k;
-            if (c < n_col) {
-              float v[8], v2[8];
-#pragma unroll
-              for (int i = 0; i < 8; ++i) {
-                v[i] = sum[k + i];
-                v2[i] = sum[(k + kHalf + i) % kSums];
-              }
-              emit8(v, v2, c, dst);
-            }
-          }
-        } else {
-          const int jstep = pool ? 2 : 1;
-          for (int j = 0, jj = 0; j < g.tiles; j += jstep, ++jj) {
-            const long long dst = dest(jj);
-            for (int c = 0; c < n_col; c += 32) {
-              float v[32], v2[32];
-              fetch(j, c, v);
-              if (pool) fetch(j + 1, c, v2);
-#pragma unroll
-              for (int i = 0; i < 32; i += 8)
-                if (c + i < n_col) {
-                  float a[8], b[8];
-#pragma unroll
-                  for (int k = 0; k < 8; ++k) {
-                    a[k] = v[i + k];
-                    b[k] = v2[i + k];
-                  }
-                  emit8(a, b, c + i, dst);
-                }
-            }
+            if (pool) pool_columns(v, v2);
+            // (a warp stores its own columns only)
+            finish_columns<HALF>(g, yv, v, bias_s, dst, it.f0, col0 + c, min(n_f, col0 + n_col), plane, pool, pairs, lane);
           }
         }
+      }
+      if (!HALF && !g.out_col) {
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        warp_arrive(bar_ce, lane);
       }
       if (HALF) {
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -1164,6 +1173,57 @@ dense_kernel(const DeviceLayer L, const __grid_constant__ DGeo g, const void* __
     if (tid == 0) T_FLUSH(7, 9);
     if (tid == 0) T_STAMP(12);
     if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");
+  }
+
+  if (g.cluster) {
+    // The CTAs of a tile share out its columns: each adds up its eight-column blocks over all of them, in
+    // rank order, and finishes them.
+    cluster_sync();
+    Item it;
+    if (warp < C::kEpiWarps && get_item(g, share, 0, &it)) {
+      uint32_t rank;
+      asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+      const int q = warp & 3, n_col = g.nt / C::kGroups, col0 = (warp >> 2) * n_col;
+      const int n_f = min(g.nt, g.c_out - it.f0);
+      const size_t plane = (size_t)g.h_out * g.w_out;
+      const bool pool = g.pool != 0;
+      const bool pairs = !pool && (g.w_out & 1) == 0 && (g.strip_w & 1) == 0;
+      const uint32_t xb = sbase + (uint32_t)g.a_off;
+      auto gather = [&](int c4, float (&v)[8]) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = 0.f;
+#pragma unroll 1
+        for (int p0 = 0; p0 < g.parts; p0 += 4) {
+          float4 a[4], b[4];
+#pragma unroll
+          for (int p = 0; p < 4; ++p)
+            if (p0 + p < g.parts) {
+              a[p] = ld_cluster(exchange_addr(xb, c4, warp, lane), (uint32_t)(p0 + p));
+              b[p] = ld_cluster(exchange_addr(xb, c4 + 1, warp, lane), (uint32_t)(p0 + p));
+            }
+#pragma unroll
+          for (int p = 0; p < 4; ++p)
+            if (p0 + p < g.parts) {
+              v[0] += a[p].x; v[1] += a[p].y; v[2] += a[p].z; v[3] += a[p].w;
+              v[4] += b[p].x; v[5] += b[p].y; v[6] += b[p].z; v[7] += b[p].w;
+            }
+        }
+      };
+      const int jstep = pool ? 2 : 1, blocks = n_col / 8;
+#pragma unroll 1
+      for (int i = (int)rank; i < g.tiles / jstep * blocks; i += g.parts) {
+        const int jj = i / blocks, c = (i - jj * blocks) * 8;
+        const long long dst = lane_dest(g, it.m0 + 128 * jj + 32 * q + lane, it.f0, plane);
+        float v[8], v2[8];
+        gather((jj * jstep * n_col + c) / 4, v);
+        if (pool) {
+          gather(((jj * jstep + 1) * n_col + c) / 4, v2);
+          pool_columns(v, v2);
+        }
+        finish_columns<HALF>(g, yv, v, bias_s, dst, it.f0, col0 + c, min(n_f, col0 + n_col), plane, pool, pairs, lane);
+      }
+    }
+    cluster_sync();      // (nobody leaves while its sums are being read)
   }
 
   // ---- common exit ----------------------------------------------------------------------------
@@ -1337,6 +1397,8 @@ bool dense_geo(const DeviceLayer& L, int n, int h, int w, bool pool, bool p8, in
   g.n_buf = (half && tiles * nt <= 256) ? 2 : 1;
   if (tiles * g.tile_cols > 512 || nt > 128 || (!half && tiles * nt > (p8 ? 256 : 128))) return false;
   if (!half && tiles > 2) return false;
+  g.out_col = !half && tiles * (g.tile_cols + nt) <= 512 ? tiles * g.tile_cols : 0;
+  g.out_stride = g.out_col ? nt : g.tile_cols;
   // the epilogue reads columns by 16, which may pass the end of a tile but not Tensor Memory's
   if (half && (g.n_buf == 2 ? 256 : 0) + (tiles - 1) * nt + nt / 2 + round_up(nt / 2, 16) > 512) return false;
   if (!half && (tiles - 1) * g.tile_cols + (g.form3 ? 2 : 1) * nt + nt / 2 + round_up(nt / 2, 16) > 512) return false;
@@ -1345,7 +1407,7 @@ bool dense_geo(const DeviceLayer& L, int n, int h, int w, bool pool, bool p8, in
   g.k_steps = (L.c_in + 15) / 16;
   g.a_bytes = pieces * 2 * g.q_tot * 16;
   g.b_bytes = g.tps * pieces * 2 * nt * 16;
-  g.a_off = round_up(kHeader + 4 * g.n_vec * (int)sizeof(Load), 128);
+  g.a_off = round_up(kHeader + kTables * g.n_vec * (int)sizeof(Load), 128);
   const int avail = kSmemLimit - g.a_off;
   // Activation stages first (two, so that one is filled while the other is read), then as many weight
   // slots as fit: what matters there is the time of the MMAs they cover against a copy's latency.
@@ -1369,7 +1431,7 @@ bool dense_geo(const DeviceLayer& L, int n, int h, int w, bool pool, bool p8, in
 size_t slots(const DGeo& g) { return std::min(g.grid, g.n_tiles); }
 size_t sums_bytes(const DGeo& g) { return slots(g) * g.tiles * g.nt * 128 * sizeof(float); }
 size_t split_bytes(const DGeo& g) {
-  return g.split ? sums_bytes(g) + ((slots(g) * 8 * sizeof(int) + 255) & ~(size_t)255) : 0;
+  return g.split && !g.cluster ? sums_bytes(g) + ((slots(g) * 8 * sizeof(int) + 255) & ~(size_t)255) : 0;
 }
 
 // Estimated cycles of a launch.  A step lasts as long as its MMAs, its share of the weight stream (about
@@ -1395,12 +1457,16 @@ double dense_cycles(const DGeo& g, bool half) {
   const double segments = std::ceil(steps / g.k_steps);
   double c = 4500 + steps * step + epi + (segments - 1) * (half && g.n_buf == 1 ? epi : 0.25 * epi);
   if (g.split) {
-    // a part adds its sums to the workspace (about 12 bytes a cycle and SM), the last one reads them back
-    const double sums = 2500 + (double)g.tiles * nt * 512 / 12.0;
-    c += sums * (g.parts ? 1.0 : 2.0) + 2000;
+    // a part hands its sums over: inside a cluster, or added to the workspace (measured: reductions of all
+    // SMs together take about 1 TB/s, and the last part waits for them before it reads the sums back)
+    const double bytes = (double)g.tiles * nt * 512;
+    if (g.cluster) c += 3500 + bytes / 24.0;
+    else c += (4000 + bytes / 6.0) * (g.parts ? 1.0 : 2.0) + 2000;
   }
   return c;
 }
+
+int max_clusters(bool half, int parts);   // below: needs the kernels
 
 // The geometry of a launch: the cheapest by the estimate.  ws_bytes: workspace the caller has.
 bool dense_plan(const DeviceLayer& L, int n, int h, int w, bool pool, bool p8, size_t ws_bytes, DGeo* out, double* cycles) {
@@ -1410,8 +1476,8 @@ bool dense_plan(const DeviceLayer& L, int n, int h, int w, bool pool, bool p8, s
   bool found = false;
   double best = 0.0;
 #ifdef PCONV_DEV
-  int force[3] = {0, 0, 0};
-  if (const char* e = getenv("PCONV_FORCE_DENSE")) sscanf(e, "%d,%d,%d", &force[0], &force[1], &force[2]);
+  int force[4] = {0, 0, 0, 0};
+  if (const char* e = getenv("PCONV_FORCE_DENSE")) sscanf(e, "%d,%d,%d,%d", &force[0], &force[1], &force[2], &force[3]);
 #endif
   int last_nt = 0;
   for (int parts = (L.dense_rows + 127) / 128; parts <= L.dense_rows / 16; parts = parts < 4 ? parts + 1 : parts * 2) {
@@ -1424,26 +1490,32 @@ bool dense_plan(const DeviceLayer& L, int n, int h, int w, bool pool, bool p8, s
       if (!dense_geo(L, n, h, w, pool, p8, tiles, nt, &g)) continue;
       // Whole tiles only; or each tile cut in `parts` equal parts (a CTA has one, and the parts of a tile end
       // together); or the line of steps cut evenly among all SMs.
-      for (int parts = 0; parts <= g.k_steps / kMinSteps + 1; ++parts) {
+      // ... or, up to eight parts, by a cluster that needs no workspace.
+      for (int v = 0; v <= 2 * (g.k_steps / kMinSteps) + 1; ++v) {
         DGeo c = g;
+        const int parts = v < 2 ? v : v / 2;
         if (parts == 1) {
-          if (g.n_tiles % sms == 0 || g.k_steps < 2 * kMinSteps) continue;
+          if (v != 1 || g.n_tiles % sms == 0 || g.k_steps < 2 * kMinSteps) continue;
           c.grid = (int)std::min<long long>(sms, (long long)g.n_tiles * (g.k_steps / kMinSteps));
           c.split = 1;
         } else if (parts > 1) {
           if ((long long)g.n_tiles * parts > sms || g.k_steps < kMinSteps * parts) break;
-          if (g.k_steps % parts != 0) continue;
           c.grid = g.n_tiles * parts;
           c.split = 1;
+          c.cluster = v & 1;
+          if (!c.cluster && g.k_steps % parts != 0) continue;
+          if (c.cluster && (parts > 8 || g.n_tiles > max_clusters(half, parts) ||
+                            tiles * nt * 512 > g.a_stages * g.a_bytes + g.b_slots * g.b_bytes))
+            continue;
         }
         if (split_bytes(c) > ws_bytes) continue;
         const int all = c.split ? c.n_tiles * c.k_steps : c.n_tiles;
         c.share = all / c.grid;
         c.share_more = all % c.grid;
-        c.parts = c.split && c.share_more == 0 && c.k_steps % c.share == 0 ? c.k_steps / c.share : 0;
+        c.parts = c.cluster ? parts : c.split && c.share_more == 0 && c.k_steps % c.share == 0 ? c.k_steps / c.share : 0;
         double cost = dense_cycles(c, half);
 #ifdef PCONV_DEV
-        if (force[0] && (force[0] != tiles || force[1] != nt || force[2] != c.grid)) cost += 1e12;
+        if (force[0] && (force[0] != tiles || force[1] != nt || force[2] != c.grid || force[3] != c.cluster)) cost += 1e12;
 #endif
         if (!found || cost < best) {
           found = true;
@@ -1484,8 +1556,8 @@ const PlanEntry& cached_plan(const DeviceLayer& L, int n, int h, int w, bool poo
     e.found = dense_plan(L, n, h, w, pool, p8, ws_bytes, &e.geo, &e.cycles);
 #ifdef PCONV_DEV
     if (e.found && getenv("PCONV_DENSE_VERBOSE"))
-      fprintf(stderr, "dense %d->%d %dx%d n%d s%d pool%d p8 %d ws%zu: tiles %d nt %d split %d grid %d n_tiles %d q %d pitch %d a_stages %d b_slots %d cycles %.0f\n",
-              L.c_in, L.c_out, h, w, n, L.stride, (int)pool, (int)p8, ws_bytes, e.geo.tiles, e.geo.nt, e.geo.split, e.geo.grid,
+      fprintf(stderr, "dense %d->%d %dx%d n%d s%d pool%d p8 %d ws%zu: tiles %d nt %d split %d cluster %d grid %d n_tiles %d q %d pitch %d a_stages %d b_slots %d cycles %.0f\n",
+              L.c_in, L.c_out, h, w, n, L.stride, (int)pool, (int)p8, ws_bytes, e.geo.tiles, e.geo.nt, e.geo.split, e.geo.cluster * e.geo.parts, e.geo.grid,
               e.geo.n_tiles, e.geo.q_tot, e.geo.pitch, e.geo.a_stages, e.geo.b_slots, e.cycles);
 #endif
     e.key = k;
@@ -1526,6 +1598,42 @@ __global__ void __launch_bounds__(128) dense_weights_kernel(const DeviceLayer L)
   }
 }
 
+// Clusters of `parts` CTAs that the device holds at once (one CTA per SM, the SMs of a cluster inside one
+// GPC); asked once per size and device.  Without a device: none.
+int max_clusters(bool half, int parts) {
+  static std::atomic<int> known[64][2][9];
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
+    cudaGetLastError();
+    return 0;
+  }
+  std::atomic<int>& slot = known[dev][half ? 1 : 0][parts];
+  int v = slot.load();
+  if (v) return v - 1;
+  const void* f = half ? (const void*)dense_kernel<true, 0> : (const void*)dense_kernel<false, 0>;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)parts, 1, 1);
+  cfg.blockDim = dim3(Cfg<false, true>::kThreads, 1, 1);
+  cfg.dynamicSmemBytes = kSmemLimit;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)parts;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&n, f, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    n = 0;
+  }
+#ifdef PCONV_DEV
+  if (getenv("PCONV_DENSE_VERBOSE")) fprintf(stderr, "clusters of %d: %d\n", parts, n);
+#endif
+  slot.store(n + 1);
+  return n;
+}
+
 template <bool HALF, int V>
 cudaError_t launch_dense_geo(const DeviceLayer& L, const DGeo& g, const void* x, const float* bias, void* y, float* ws,
                              int* tickets, cudaStream_t stream) {
@@ -1545,11 +1653,14 @@ cudaError_t launch_dense_geo(const DeviceLayer& L, const DGeo& g, const void* x,
   // more than half of an SM's shared memory: one CTA per SM (each takes all of Tensor Memory)
   cfg.dynamicSmemBytes = (size_t)(smem < 120 * 1024 ? 120 * 1024 : smem);
   cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)g.parts;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = g.cluster ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, dense_kernel<HALF, V>, L, g, x, bias, y, ws, tickets);
 }
 
