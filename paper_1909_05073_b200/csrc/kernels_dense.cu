@@ -1456,12 +1456,16 @@ double dense_cycles(const DGeo& g, bool half) {
                                : std::ceil((double)g.n_tiles / g.grid) * g.k_steps;
   const double segments = std::ceil(steps / g.k_steps);
   double c = 4500 + steps * step + epi + (segments - 1) * (half && g.n_buf == 1 ? epi : 0.25 * epi);
+  // One CTA per SM: up to half of the SMs, a launch sets itself up while the one before it still runs.
+  if (2 * g.grid > sms) c += 2500;
   if (g.split) {
-    // a part hands its sums over: inside a cluster, or added to the workspace (measured: reductions of all
-    // SMs together take about 1 TB/s, and the last part waits for them before it reads the sums back)
+    // A part hands its sums over, inside a cluster or added to the workspace.  Measured on layers of 49 to
+    // 3136 positions: a cluster's exchange 5000-6000 cycles, more where large clusters have to wait for
+    // neighbouring SMs; the workspace's about as much up to some 30 KB per SM, then reductions of all SMs
+    // together run at about 1 TB/s.  An uneven split goes through it twice.
     const double bytes = (double)g.tiles * nt * 512;
-    if (g.cluster) c += 3500 + bytes / 24.0;
-    else c += (4000 + bytes / 6.0) * (g.parts ? 1.0 : 2.0) + 2000;
+    if (g.cluster) c += 4700 + bytes / 24.0 + (g.parts > 4 ? 800.0 : 0.0) + (g.parts >= 4 && 2 * g.grid > sms ? 1500.0 : 0.0);
+    else c += (4200 + bytes * g.grid / sms / 8.0) * (g.parts ? 1.0 : 2.0);
   }
   return c;
 }
