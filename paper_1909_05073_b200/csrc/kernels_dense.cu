@@ -1435,7 +1435,7 @@ size_t split_bytes(const DGeo& g) {
 }
 
 // Estimated cycles of a launch.  A step lasts as long as its MMAs, its share of the weight stream (about
-// 24 bytes a cycle and SM from L2) or the staging of its activations, whichever is longest; an item ends with its stores, which only the fp32 kernel
+// 36 bytes a cycle and SM from L2) or the staging of its activations, whichever is longest; an item ends with its stores, which only the fp32 kernel
 // and two accumulator sets overlap with the next item; a split adds the exchange of partial sums.
 double dense_cycles(const DGeo& g, bool half) {
   const double sms = device_sm_count();
@@ -1444,7 +1444,7 @@ double dense_cycles(const DGeo& g, bool half) {
                     : (g.form3 ? mma_cycles(3 * nt) + mma_cycles(2 * nt) + mma_cycles(nt)
                                : mma_cycles(2 * nt) + 4 * mma_cycles(nt));
   double step = tap * g.n_taps * g.tiles;
-  const double wb = ((double)g.n_taps * (half ? 1 : 3) * nt * 32 + (g.vec ? 0.0 : g.a_bytes)) / 24.0;
+  const double wb = ((double)g.n_taps * (half ? 1 : 3) * nt * 32 + (g.vec ? 0.0 : g.a_bytes)) / 36.0;
   // (a batch of the producers -- a load and its rows a thread -- takes about as long whatever its width)
   double conv = 300.0 + (half ? 1100.0 : 1300.0) * ((2 * g.n_vec + 319) / 320);
   if (!g.vec) conv = 60.0 * (half ? 2 : 6) * g.planes;      // one bulk copy each
@@ -1751,15 +1751,16 @@ cudaError_t launch_dense(const DeviceLayer& L, const void* x, const float* bias,
   return launch_dense_geo<false, 1>(L, g, x, bias, y, sums, tickets, stream);
 }
 
-// What is expected to run this shape fastest: both kernels by estimate.  Sparse kernel: a fixed 12 us and
-// a fifth of the FP32 peak (measured on the benchmark's layers: 15-29 % of it in large launches).  Dense
+// What is expected to run this shape fastest: both kernels by estimate.  Sparse kernel: a fixed 12 us, 12 ns a
+// channel (measured at 1 image: 14-15 us at 64-128 channels, 18-23 us at 512) and a fifth of the FP32 peak
+// (15-29 % of it in large launches).  Dense
 // kernel: measured times are 1.3-1.45 times the estimated cycles at the full clock, of which the clock under
 // tensor load (1.65 of 1.9 GHz) is the larger part.  Staging the input as position rows is a launch of its
 // own and moves every value twice.
 DensePath dense_path(const DeviceLayer& L, int n, int h, int w, bool pool, RowsFrom rows, size_t ws_bytes) {
   const bool half = L.storage == PCONV_F16;
   const double macs = 4.0 * (double)L.n_kept * n * ((h - 1) / L.stride + 1) * ((w - 1) / L.stride + 1);
-  double best = 1380.0 * (12.0 + 2.0 * macs / (0.2 * 74.45e6));
+  double best = 1380.0 * (12.0 + 0.012 * L.c_in + 2.0 * macs / (0.2 * 74.45e6));
   DensePath path = kNotDense;
 #ifdef PCONV_DEV
   if (getenv("PCONV_FORCE_DENSE")) best = 1e15;
