@@ -489,17 +489,22 @@ __device__ __forceinline__ void store_rows(void* __restrict__ y, const DGeo& g, 
   }
 }
 
-// Bias, ReLU and store of eight finished columns (filters f0 + col ..) of this lane's position.
+// Bias and ReLU of eight finished columns.
+__device__ __forceinline__ void add_bias(float (&v)[8], const float* bias, bool relu) {
+  const float4 a = reinterpret_cast<const float4*>(bias)[0], b = reinterpret_cast<const float4*>(bias)[1];
+  v[0] += a.x; v[1] += a.y; v[2] += a.z; v[3] += a.w;
+  v[4] += b.x; v[5] += b.y; v[6] += b.z; v[7] += b.w;
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    if (relu) v[i] = fmaxf(v[i], 0.f);
+}
+// ... and their store (filters f0 + col ..) at this lane's position.
 template <bool HALF>
 __device__ __forceinline__ void finish_columns(const DGeo& g, void* __restrict__ y, float (&v)[8], const float* bias_s,
                                                long long dst, int f0, int col, int n_f, size_t plane, bool pool,
                                                bool pairs, int lane) {
   typedef typename std::conditional<HALF, __half, float>::type T;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    v[i] += bias_s[(col + i) & 127];
-    if (g.relu) v[i] = fmaxf(v[i], 0.f);
-  }
+  add_bias(v, bias_s + col, g.relu);
   if (g.out_p8) {
     // (the last filter tile may reach past the layer's filters, and so past the next layer's groups)
     if (f0 + col < g.rows) store_rows<HALF>(y, g, v, dst, (f0 + col) >> 3, pool, lane);
@@ -1138,24 +1143,39 @@ dense_kernel(const DeviceLayer L, const __grid_constant__ DGeo g, const void* __
       }
       const long long t_fin = T_NOW();
       if (finish) {
+        // kWide columns at a time: the loads, conversions and stores of a block overlap, and what 8 warps
+        // cannot hide of each other's latency is waited for once a block.
+        constexpr int kWide = HALF ? 32 : 16;
         const int jstep = pool ? 2 : 1;
         for (int j = 0, jj = 0; j < g.tiles; j += jstep, ++jj) {
           const long long dst = lane_dest(g, it.m0 + 128 * jj + 32 * q + lane, it.f0, plane);
+          const uint32_t from = res + (uint32_t)j * res_stride;
 #pragma unroll 1
-          for (int c = 0; c < n_col; c += 8) {
-            uint32_t r[8], r2[8];
-            tmem_ld8(r, res + (uint32_t)j * res_stride + (uint32_t)c);
-            if (pool) tmem_ld8(r2, res + (uint32_t)(j + 1) * res_stride + (uint32_t)c);
-            tmem_ld_wait();
-            float v[8], v2[8];
+          for (int c = 0; c < n_col; c += kWide) {
+            uint32_t r[kWide / 8][8];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              v[i] = __uint_as_float(r[i]);
-              v2[i] = __uint_as_float(r2[i]);
+            for (int k = 0; k < kWide / 8; ++k)
+              if (c + 8 * k < n_col) tmem_ld8(r[k], from + (uint32_t)(c + 8 * k));
+            tmem_ld_wait();
+#pragma unroll
+            for (int k = 0; k < kWide / 8; ++k) {
+              if (c + 8 * k >= n_col) break;
+              float v[8];
+#pragma unroll
+              for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[k][i]);
+              if (pool) {
+                uint32_t r2[8];
+                float v2[8];
+                tmem_ld8(r2, from + res_stride + (uint32_t)(c + 8 * k));
+                tmem_ld_wait();
+#pragma unroll
+                for (int i = 0; i < 8; ++i) v2[i] = __uint_as_float(r2[i]);
+                pool_columns(v, v2);
+              }
+              // (a warp stores its own columns only)
+              finish_columns<HALF>(g, yv, v, bias_s, dst, it.f0, col0 + c + 8 * k, min(n_f, col0 + n_col), plane, pool,
+                                   pairs, lane);
             }
-            if (pool) pool_columns(v, v2);
-            // (a warp stores its own columns only)
-            finish_columns<HALF>(g, yv, v, bias_s, dst, it.f0, col0 + c, min(n_f, col0 + n_col), plane, pool, pairs, lane);
           }
         }
       }
