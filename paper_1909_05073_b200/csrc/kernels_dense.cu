@@ -102,6 +102,8 @@ struct DGeo {
   int n_tiles, grid;                 // (positions, filters) tiles, CTAs
   int cluster;                       // the CTAs of a tile are a thread-block cluster and exchange their sums directly
   int share, share_more, parts;      // a CTA's tiles or steps (the first share_more: one more); equal parts of a tile
+  uint32_t cell_mul, pitch_mul;      // p / cell_pos and p / pitch by multiplication, then shifts (see fast_div)
+  int cell_shift, pitch_shift;
   int in_plane_len, in_lead;         // P8 source: positions of a plane, positions before the batch's first
   int out_p8, out_pitch, out_cell_rows, out_sy, out_sx, out_plane_len, out_lead;   // P8 result: the next layer's rows
   int tap_off[kMaxT][9];             // start position of (tile, stored tap) inside a staged slab
@@ -399,13 +401,24 @@ __device__ __forceinline__ void store_position(uint32_t dst, uint32_t slab, cons
   }
 }
 
+// p / d for 0 <= p < 2^31 and d >= 2 (a division by a run-time number is some 150 cycles, and a lane's
+// position takes two a tile): with 2^(l-1) < d <= 2^l and mul = floor(2^(31+l) / d) + 1, mul * d exceeds
+// 2^(31+l) by at most 2^l, too little to reach the next quotient.
+__device__ __forceinline__ int fast_div(int p, uint32_t mul, int shift) { return (int)(__umulhi((uint32_t)p, mul) >> shift); }
+void fast_div_of(int d, uint32_t* mul, int* shift) {
+  int l = 1;
+  while ((1ll << l) < d) ++l;
+  *mul = (uint32_t)((1ull << (31 + l)) / (unsigned)d + 1);
+  *shift = l - 1;
+}
+
 // Where a lane's position goes in y: element offset of filter 0, or -1 if nothing is stored there.
 __device__ __forceinline__ long long position_dest(const DGeo& g, int p) {
-  const int cell = p / g.cell_pos;
+  const int cell = fast_div(p, g.cell_mul, g.cell_shift);
   if (cell >= g.n_cells) return -1;
   const int r = p - cell * g.cell_pos;
-  const int i = r / g.pitch, j = r - i * g.pitch;
-  const int img = cell / g.strips, st = cell - img * g.strips;
+  const int i = fast_div(r, g.pitch_mul, g.pitch_shift), j = r - i * g.pitch;
+  const int img = g.strips == 1 ? cell : cell / g.strips, st = cell - img * g.strips;
   int col = st * g.strip_w + j;
   if (j >= g.strip_w) return -1;
   if (g.pool) col >>= 1;
@@ -426,39 +439,60 @@ __device__ __forceinline__ void store_chunk(float* __restrict__ y, const float (
                                             size_t plane, bool pool, bool, int lane) {
   if (dst < 0) return;
   float* p = y + dst + (size_t)c * plane;
+  const int room = n_f - c;
   if (pool) {
-    if (lane & 1) p += plane;
+    const bool odd = lane & 1;
+    if (odd) p += plane;
 #pragma unroll
     for (int i = 0; i < 8; i += 2, p += 2 * plane)
-      if (c + i + (lane & 1) < n_f) *p = (lane & 1) ? v[i + 1] : v[i];
+      if (i + (lane & 1) < room) *p = odd ? v[i + 1] : v[i];
+  } else if (room >= 8) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i, p += plane) *p = v[i];
   } else {
 #pragma unroll
     for (int i = 0; i < 8; ++i, p += plane)
-      if (c + i < n_f) *p = v[i];
+      if (i < room) *p = v[i];
   }
 }
 // fp16: where rows are an even number of columns, the two lanes of a pair exchange a value so that
 // each stores both columns of one filter (4 bytes).
 __device__ __forceinline__ void store_chunk(__half* __restrict__ y, const float (&v)[8], long long dst, int c, int n_f,
                                             size_t plane, bool pool, bool pairs, int lane) {
+  const int odd = lane & 1, room = n_f - c;
+  __half2 own[4];                                            // filters i, i + 1 at this lane's position
 #pragma unroll
-  for (int i = 0; i < 8; i += 2) {
-    const __half2 own = __floats2half2_rn(v[i], v[i + 1]);   // filters i, i + 1 at this lane's position
-    if (pool) {
-      const int f = i + (lane & 1);
-      if (dst >= 0 && c + f < n_f) y[dst + (size_t)(c + f) * plane] = (lane & 1) ? __high2half(own) : __low2half(own);
-    } else if (pairs) {
-      const uint32_t o = *reinterpret_cast<const uint32_t*>(&own);
+  for (int i = 0; i < 4; ++i) own[i] = __floats2half2_rn(v[2 * i], v[2 * i + 1]);
+  if (pool) {
+    if (dst < 0) return;
+    __half* p = y + dst + (size_t)(c + odd) * plane;
+#pragma unroll
+    for (int i = 0; i < 8; i += 2, p += 2 * plane)
+      if (i + odd < room) *p = odd ? __high2half(own[i / 2]) : __low2half(own[i / 2]);
+  } else if (pairs) {
+    uint32_t w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint32_t o = *reinterpret_cast<const uint32_t*>(&own[i]);
       const uint32_t got = __shfl_xor_sync(0xffffffffu, o, 1);
       // even lane: filter i of columns (own, next); odd lane: filter i + 1 of columns (previous, own)
-      const uint32_t w = (lane & 1) ? __byte_perm(got, o, 0x7632) : __byte_perm(o, got, 0x5410);
-      const int f = i + (lane & 1);
-      if (dst >= 0 && c + f < n_f)
-        *reinterpret_cast<uint32_t*>(y + dst - (lane & 1) + (size_t)(c + f) * plane) = w;
-    } else if (dst >= 0) {
-      if (c + i < n_f) y[dst + (size_t)(c + i) * plane] = __low2half(own);
-      if (c + i + 1 < n_f) y[dst + (size_t)(c + i + 1) * plane] = __high2half(own);
+      w[i] = odd ? __byte_perm(got, o, 0x7632) : __byte_perm(o, got, 0x5410);
     }
+    if (dst < 0) return;
+    __half* p = y + dst - odd + (size_t)(c + odd) * plane;
+    if (room >= 8) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i, p += 2 * plane) *reinterpret_cast<uint32_t*>(p) = w[i];
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i, p += 2 * plane)
+        if (2 * i + odd < room) *reinterpret_cast<uint32_t*>(p) = w[i];
+    }
+  } else if (dst >= 0) {
+    __half* p = y + dst + (size_t)c * plane;
+#pragma unroll
+    for (int i = 0; i < 8; ++i, p += plane)
+      if (i < room) *p = i & 1 ? __high2half(own[i / 2]) : __low2half(own[i / 2]);
   }
 }
 
@@ -1362,6 +1396,8 @@ bool dense_geo(const DeviceLayer& L, int n, int h, int w, bool pool, bool p8, in
   g.cell_rows = g.h_out + 1;
   g.cell_pos = g.cell_rows * g.pitch;
   g.n_cells = n * g.strips;
+  fast_div_of(g.cell_pos, &g.cell_mul, &g.cell_shift);
+  fast_div_of(g.pitch, &g.pitch_mul, &g.pitch_shift);
   g.sy = (s == 2 || pool) ? 2 : 1;
   g.sx = s;
   g.planes = s == 2 ? 4 : (pool ? 2 : 1);
