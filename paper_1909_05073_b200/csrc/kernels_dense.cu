@@ -532,14 +532,16 @@ __device__ __forceinline__ void add_bias(float (&v)[8], const float* bias, bool 
   for (int i = 0; i < 8; ++i)
     if (relu) v[i] = fmaxf(v[i], 0.f);
 }
-// ... and their store (filters f0 + col ..) at this lane's position.
-template <bool HALF>
+// ... and their store (filters f0 + col ..) at this lane's position, as position rows or NCHW (kEither: as
+// the launch says).
+enum Form { kNchw, kRows, kEither };
+template <bool HALF, Form FORM>
 __device__ __forceinline__ void finish_columns(const DGeo& g, void* __restrict__ y, float (&v)[8], const float* bias_s,
                                                long long dst, int f0, int col, int n_f, size_t plane, bool pool,
                                                bool pairs, int lane) {
   typedef typename std::conditional<HALF, __half, float>::type T;
   add_bias(v, bias_s + col, g.relu);
-  if (g.out_p8) {
+  if (FORM == kRows || (FORM == kEither && g.out_p8)) {
     // (the last filter tile may reach past the layer's filters, and so past the next layer's groups)
     if (f0 + col < g.rows) store_rows<HALF>(y, g, v, dst, (f0 + col) >> 3, pool, lane);
   } else {
@@ -558,6 +560,41 @@ __device__ __forceinline__ void pool_columns(float (&v)[8], const float (&v2)[8]
   for (int i = 0; i < 8; ++i) {
     v[i] = fmaxf(v[i], v2[i]);
     v[i] = fmaxf(v[i], __shfl_xor_sync(0xffffffffu, v[i], 1));
+  }
+}
+
+// A warp's finished columns of one tile from Tensor Memory to the result.
+template <bool HALF, Form FORM>
+__device__ __forceinline__ void emit_columns(const DGeo& g, void* __restrict__ y, uint32_t from, uint32_t tile_stride,
+                                             const float* bias_s, long long dst, int f0, int col0, int n_col, int n_f,
+                                             size_t plane, bool pool, bool pairs, int lane) {
+  constexpr int kWide = HALF && FORM == kNchw ? 8 : 16;
+#pragma unroll 1
+  for (int c = 0; c < n_col; c += kWide) {
+    uint32_t r[kWide / 8][8];
+#pragma unroll
+    for (int k = 0; k < kWide / 8; ++k)
+      if (c + 8 * k < n_col) tmem_ld8(r[k], from + (uint32_t)(c + 8 * k));
+    tmem_ld_wait();
+#pragma unroll
+    for (int k = 0; k < kWide / 8; ++k) {
+      if (c + 8 * k >= n_col) break;
+      float v[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[k][i]);
+      if (pool) {
+        uint32_t r2[8];
+        float v2[8];
+        tmem_ld8(r2, from + tile_stride + (uint32_t)(c + 8 * k));
+        tmem_ld_wait();
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v2[i] = __uint_as_float(r2[i]);
+        pool_columns(v, v2);
+      }
+      // (a warp stores its own columns only)
+      finish_columns<HALF, FORM>(g, y, v, bias_s, dst, f0, col0 + c + 8 * k, min(n_f, col0 + n_col), plane, pool, pairs,
+                                 lane);
+    }
   }
 }
 
@@ -1177,40 +1214,17 @@ dense_kernel(const DeviceLayer L, const __grid_constant__ DGeo g, const void* __
       }
       const long long t_fin = T_NOW();
       if (finish) {
-        // kWide columns at a time: the loads, conversions and stores of a block overlap, and what 8 warps
-        // cannot hide of each other's latency is waited for once a block.
-        constexpr int kWide = HALF ? 32 : 16;
+        // fp16: one loop for each form of the result, each as short as it can be: eight warps cannot hide much
+        // of each other's latency, and these loops run beside the other roles' code in small instruction caches
+        // (one loop with both forms in it took 1.2-1.4 times as long).  In the fp32 kernel, whose register sums
+        // leave no room, two loops cost spills in the channel loop and a fifth of its time.
         const int jstep = pool ? 2 : 1;
         for (int j = 0, jj = 0; j < g.tiles; j += jstep, ++jj) {
           const long long dst = lane_dest(g, it.m0 + 128 * jj + 32 * q + lane, it.f0, plane);
           const uint32_t from = res + (uint32_t)j * res_stride;
-#pragma unroll 1
-          for (int c = 0; c < n_col; c += kWide) {
-            uint32_t r[kWide / 8][8];
-#pragma unroll
-            for (int k = 0; k < kWide / 8; ++k)
-              if (c + 8 * k < n_col) tmem_ld8(r[k], from + (uint32_t)(c + 8 * k));
-            tmem_ld_wait();
-#pragma unroll
-            for (int k = 0; k < kWide / 8; ++k) {
-              if (c + 8 * k >= n_col) break;
-              float v[8];
-#pragma unroll
-              for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[k][i]);
-              if (pool) {
-                uint32_t r2[8];
-                float v2[8];
-                tmem_ld8(r2, from + res_stride + (uint32_t)(c + 8 * k));
-                tmem_ld_wait();
-#pragma unroll
-                for (int i = 0; i < 8; ++i) v2[i] = __uint_as_float(r2[i]);
-                pool_columns(v, v2);
-              }
-              // (a warp stores its own columns only)
-              finish_columns<HALF>(g, yv, v, bias_s, dst, it.f0, col0 + c + 8 * k, min(n_f, col0 + n_col), plane, pool,
-                                   pairs, lane);
-            }
-          }
+          if constexpr (!HALF) emit_columns<HALF, kEither>(g, yv, from, res_stride, bias_s, dst, it.f0, col0, n_col, n_f, plane, pool, pairs, lane);
+          else if (g.out_p8) emit_columns<HALF, kRows>(g, yv, from, res_stride, bias_s, dst, it.f0, col0, n_col, n_f, plane, pool, pairs, lane);
+          else emit_columns<HALF, kNchw>(g, yv, from, res_stride, bias_s, dst, it.f0, col0, n_col, n_f, plane, pool, pairs, lane);
         }
       }
       if (!HALF && !g.out_col) {
@@ -1274,7 +1288,8 @@ dense_kernel(const DeviceLayer L, const __grid_constant__ DGeo g, const void* __
           gather(((jj * jstep + 1) * n_col + c) / 4, v2);
           pool_columns(v, v2);
         }
-        finish_columns<HALF>(g, yv, v, bias_s, dst, it.f0, col0 + c, min(n_f, col0 + n_col), plane, pool, pairs, lane);
+        const int top = min(n_f, col0 + n_col);
+        finish_columns<HALF, kEither>(g, yv, v, bias_s, dst, it.f0, col0 + c, top, plane, pool, pairs, lane);
       }
     }
     cluster_sync();      // (nobody leaves while its sums are being read)
