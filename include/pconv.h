@@ -109,14 +109,16 @@ enum {
                                  takes ~2 us to land here and the raw ring is two deep: the first
                                  chunk is ready after 8.7-15 us against 4.3-5.6 us; 0.57 against
                                  0.38 ms for the stack). */
-  PCONV_KERNEL_TENSOR = 0x800u /* fp16 storage, stride 1 only: the layer as a dense implicit GEMM over
-                                  the zero-inserted weights on the tensor cores (tcgen05.mma, fp32
-                                  accumulators in Tensor Memory).  It multiplies the pruned zeros too
-                                  -- 9 / (4 x keep rate) times the surviving multiply-adds -- and is
-                                  still several times faster for fp16 at the benchmark's keep rates,
-                                  so the library picks it by default when the batch gives it enough
-                                  tiles; fp16 products are exact in fp32, so the result differs from
-                                  the sparse kernels by summation order only.  No fused max-pool. */
+  PCONV_KERNEL_TENSOR = 0x800u /* the layer as a dense implicit GEMM over the zero-inserted weights on
+                                  the tensor cores (tcgen05.mma, fp32 accumulators in Tensor Memory).
+                                  It multiplies the pruned zeros too -- 9 / (4 x keep rate) times the
+                                  surviving multiply-adds, for fp32 storage six times that (three exact
+                                  bf16 pieces a value, six products) -- and is still faster wherever
+                                  there is enough work for them, so the library picks it by estimate.
+                                  fp16 products are exact in fp32; the fp32 form drops less than 2^-24 of
+                                  a product.  A result differs from the sparse kernels' by summation
+                                  order, and where an activation is infinite or not a number: its
+                                  product with a pruned weight's zero is then not a number. */
 };
 
 #define PCONV_MAX_PATTERNS 16
@@ -281,9 +283,10 @@ typedef struct pconv_plan_t {
                             loads for fp16), 1 = fp16 pairs by cp.async into a raw ring, 2 / 3 = fp32 rows /
                             plane spans by bulk copies (cp.async.bulk) into a raw ring; the raw ring is
                             rebuilt into the kernel's tile layout by the producer warps */
-  int tensor_path;       /* 1 = a default forward of this shape (no kernel-selection flag, no fused
-                            pool) runs the dense tensor-core kernel instead of the tiled one; the
-                            fields above still describe the tiled kernel */
+  int tensor_path;       /* 1 = fp16 storage, stride 1, and a batch that gives the tensor cores enough
+                            tiles: a default forward of this shape (no kernel-selection flag, no fused
+                            pool) runs the dense tensor-core kernel.  Other shapes run whichever kernel
+                            is estimated to be faster; the fields above still describe the tiled one */
 } pconv_plan_t;
 
 /* Test / tuning aid: fills *plan with the geometry a tiled forward of this shape would use;

@@ -33,11 +33,22 @@
 //  * Cost of one MMA of 128 x N x 16: max(N / 2, 32 + N / 4) cycles (measured; the second term is its
 //    operands at 128 bytes a cycle from shared memory).  Pieces of the weights are therefore stacked
 //    along N where one A operand meets several of them.
-//  * Warps: 16 (fp32) or 8 (fp16) epilogue warps, one that issues the MMAs, one that streams weights
-//    through a ring, 4 or 8 that load activations from NCHW, convert and store them.  One persistent CTA
-//    per SM.
-//  * Few tiles: channel steps are cut into parts that different CTAs take; partial sums meet in the
-//    caller's workspace (16-byte vector reductions, a ticket per warp's part; the last one finishes).
+//  * Warps: 8 epilogue warps, one that issues the MMAs, one that streams weights through a ring, and
+//    either 10 that load activations from NCHW, convert and store them, or one that copies them where they
+//    come as position rows (below).  One persistent CTA per SM.
+//  * Position rows.  Between the layers of a stack, and where the caller has memory for them, activations
+//    lie in global memory as the tensor core reads them, split into pieces already: bulk copies replace
+//    the producers' loads and conversions (256->256 56x56 fp32 N=1: 37 us against 33).
+//  * Few tiles: channel steps are cut into parts that different CTAs take.  Up to eight CTAs of a tile form
+//    a cluster and add their sums up through distributed shared memory, in rank order; otherwise partial
+//    sums meet in the caller's workspace (16-byte vector reductions, a ticket per warp's part; the last
+//    one finishes).
+//  * Instruction caches.  The roles run different code side by side, so every loop is kept short: the
+//    epilogue unrolled over its registers took 10 us a tile to fetch, a wait loop unrolled by the compiler
+//    half of the kernel's speed.
+//  * What bounds it: the tensor pipe in large fp32 launches (512->512 14x14 N=64: 589 us in the sparse
+//    kernel, 326 here); with 64 filters or few channels the epilogue; at one image a fixed 9-10 us of
+//    launch, first copies and exchange, then the weight stream (36 bytes a cycle and SM from L2).
 //  * Every wait is bounded; one that runs out records its id in the status word, the role stops
 //    working, and all roles meet at the common exit where Tensor Memory is released.
 #include <cuda_fp16.h>
@@ -1506,8 +1517,9 @@ size_t split_bytes(const DGeo& g) {
 }
 
 // Estimated cycles of a launch.  A step lasts as long as its MMAs, its share of the weight stream (about
-// 36 bytes a cycle and SM from L2) or the staging of its activations, whichever is longest; an item ends with its stores, which only the fp32 kernel
-// and two accumulator sets overlap with the next item; a split adds the exchange of partial sums.
+// 36 bytes a cycle and SM from L2) or the staging of its activations, whichever is longest; an item ends with
+// its stores, which only the fp32 kernel and two accumulator sets overlap with the next item; a split adds
+// the exchange of partial sums.
 double dense_cycles(const DGeo& g, bool half) {
   const double sms = device_sm_count();
   const int nt = g.nt;
@@ -1563,9 +1575,9 @@ bool dense_plan(const DeviceLayer& L, int n, int h, int w, bool pool, bool p8, s
     for (int tiles = 1; tiles <= kMaxT; tiles *= 2) {
       DGeo g;
       if (!dense_geo(L, n, h, w, pool, p8, tiles, nt, &g)) continue;
-      // Whole tiles only; or each tile cut in `parts` equal parts (a CTA has one, and the parts of a tile end
-      // together); or the line of steps cut evenly among all SMs.
-      // ... or, up to eight parts, by a cluster that needs no workspace.
+      // Whole tiles only (v = 0); or the line of steps cut evenly among all SMs (1); or each tile cut in
+      // v / 2 parts, a CTA's each: in the workspace (even v; equal parts, which end together) or, up to
+      // eight, by a cluster, which needs none.
       for (int v = 0; v <= 2 * (g.k_steps / kMinSteps) + 1; ++v) {
         DGeo c = g;
         const int parts = v < 2 ? v : v / 2;
@@ -1824,10 +1836,9 @@ cudaError_t launch_dense(const DeviceLayer& L, const void* x, const float* bias,
 
 // What is expected to run this shape fastest: both kernels by estimate.  Sparse kernel: a fixed 12 us, 12 ns a
 // channel (measured at 1 image: 14-15 us at 64-128 channels, 18-23 us at 512) and a fifth of the FP32 peak
-// (15-29 % of it in large launches).  Dense
-// kernel: measured times are 1.3-1.45 times the estimated cycles at the full clock, of which the clock under
-// tensor load (1.65 of 1.9 GHz) is the larger part.  Staging the input as position rows is a launch of its
-// own and moves every value twice.
+// (15-29 % of it in large launches).  Dense kernel: measured times are 1.3-1.45 times the estimated cycles at
+// the full clock, of which the clock under tensor load (1.65 of 1.9 GHz) is the larger part.  Staging the
+// input as position rows is a launch of its own and moves every value twice.
 DensePath dense_path(const DeviceLayer& L, int n, int h, int w, bool pool, RowsFrom rows, size_t ws_bytes) {
   const bool half = L.storage == PCONV_F16;
   const double macs = 4.0 * (double)L.n_kept * n * ((h - 1) / L.stride + 1) * ((w - 1) / L.stride + 1);
