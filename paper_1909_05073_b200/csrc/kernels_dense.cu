@@ -1540,8 +1540,6 @@ double dense_cycles(const DGeo& g, bool half) {
                                : std::ceil((double)g.n_tiles / g.grid) * g.k_steps;
   const double segments = std::ceil(steps / g.k_steps);
   double c = 4500 + steps * step + epi + (segments - 1) * (half && g.n_buf == 1 ? epi : 0.25 * epi);
-  // One CTA per SM: up to half of the SMs, a launch sets itself up while the one before it still runs.
-  if (2 * g.grid > sms) c += 2500;
   if (g.split) {
     // A part hands its sums over, inside a cluster or added to the workspace.  Measured on layers of 49 to
     // 3136 positions: a cluster's exchange 5000-6000 cycles, more where large clusters have to wait for
@@ -1630,8 +1628,8 @@ struct PlanEntry {
   double cycles;
   DGeo geo;
 };
-// Eight entries a set, the oldest replaced: with one entry a set, a few of the thirty keys of a 16-layer
-// network always met, and each pass planned those again (ResNet-50 N=1: 309 us a pass, 210 of them kernels).
+// Eight entries a set, the oldest replaced: with one entry a set, a few of the 48 keys of a 16-layer
+// network always met, and each pass planned those again (ResNet-50 N=1: 309 us a pass, now 268).
 const PlanEntry& cached_plan(const DeviceLayer& L, int n, int h, int w, bool pool, bool p8, size_t ws_bytes) {
   constexpr int kSets = 64, kWays = 8;
   struct Table {
@@ -1869,7 +1867,7 @@ DensePath dense_path(const DeviceLayer& L, int n, int h, int w, bool pool, RowsF
     const PlanEntry& e = cached_plan(L, n, h, w, pool, true, ws_bytes);
     double cycles = e.cycles;
     if (e.found && rows == kRowsStaged)
-      cycles += 3500.0 + ((double)rows_bytes(rows_of(L.c_in, L.stride, n, h, w, pool), half) +
+      cycles += 5500.0 + ((double)rows_bytes(rows_of(L.c_in, L.stride, n, h, w, pool), half) +
                           (double)n * L.c_in * h * w * (half ? 2 : 4)) / 2200.0;
     if (e.found && cycles < best) path = kFromRows;
   }
