@@ -1842,30 +1842,36 @@ cudaError_t launch_dense(const DeviceLayer& L, const void* x, const float* bias,
   return launch_dense_geo<false, 1>(L, g, x, bias, y, sums, tickets, stream);
 }
 
-// What is expected to run this shape fastest: both kernels by estimate.  Sparse kernel: a fixed 12 us, 12 ns a
-// channel (measured at 1 image: 14-15 us at 64-128 channels, 18-23 us at 512) and a fifth of the FP32 peak
-// (15-29 % of it in large launches).  Dense kernel: measured times are 1.3-1.45 times the estimated cycles at
-// the full clock, of which the clock under tensor load (1.65 of 1.9 GHz) is the larger part.  Staging the
-// input as position rows is a launch of its own and moves every value twice.
+// What is expected to run this shape fastest: both kernels by estimate.  Sparse kernel: a fixed 12 us, 8 ns a
+// channel, twice that at stride 2 (measured at 1 image: 14-15 us at 64-128 channels, 18-23 us at 512) and a
+// fifth of the FP32 peak (15-29 % of it in large launches).  Dense kernel: measured times are 1.3-1.45 times
+// the estimated cycles at the full clock, of which the clock under tensor load (1.65 of 1.9 GHz) is the larger
+// part.  Staging the input as position rows is a launch of its own and moves every value twice.  Where a
+// tile's positions are all there are, each dense weight (54 bytes for fp32, a kept kernel's sparse ones take 6
+// a weight) is read for one use and, in a network of such layers, from memory: 512->512 7x7 takes 15 us alone
+// and 20-26 us among its neighbours, the sparse kernel 18 us in both.
 DensePath dense_path(const DeviceLayer& L, int n, int h, int w, bool pool, RowsFrom rows, size_t ws_bytes) {
   const bool half = L.storage == PCONV_F16;
   const double macs = 4.0 * (double)L.n_kept * n * ((h - 1) / L.stride + 1) * ((w - 1) / L.stride + 1);
-  double best = 1380.0 * (12.0 + 0.012 * L.c_in + 2.0 * macs / (0.2 * 74.45e6));
+  double best = 1380.0 * (12.0 + 0.008 * L.c_in * L.stride + 2.0 * macs / (0.2 * 74.45e6));
   DensePath path = kNotDense;
+  auto cycles_of = [&](const PlanEntry& e) {
+    return e.cycles + (e.geo.n_tiles <= e.geo.n_ft ? (double)dense_weight_bytes(L) / 1600.0 : 0.0);
+  };
 #ifdef PCONV_DEV
   if (getenv("PCONV_FORCE_DENSE")) best = 1e15;
   if (const char* f = getenv("PCONV_FORCE_ROWS")) rows = atoi(f) && rows != kNoRows ? kRowsGiven : kNoRows;
 #endif
   if (rows != kRowsGiven) {
     const PlanEntry& e = cached_plan(L, n, h, w, pool, false, ws_bytes);
-    if (e.found && e.cycles < best) {
-      best = e.cycles;
+    if (e.found && cycles_of(e) < best) {
+      best = cycles_of(e);
       path = kFromNchw;
     }
   }
   if (rows != kNoRows) {
     const PlanEntry& e = cached_plan(L, n, h, w, pool, true, ws_bytes);
-    double cycles = e.cycles;
+    double cycles = cycles_of(e);
     if (e.found && rows == kRowsStaged)
       cycles += 5500.0 + ((double)rows_bytes(rows_of(L.c_in, L.stride, n, h, w, pool), half) +
                           (double)n * L.c_in * h * w * (half ? 2 : 4)) / 2200.0;
