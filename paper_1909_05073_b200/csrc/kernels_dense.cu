@@ -381,13 +381,20 @@ __device__ __forceinline__ uint32_t bf16_pair(float a, float b) {
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
   return r;
 }
+// The same with what would round to infinity (from 3.396e38 on) as the largest finite value.
+__device__ __forceinline__ uint32_t bf16_pair_sat(float a, float b) {
+  uint32_t r;
+  asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
+  return r;
+}
 // Two fp32 values as three bf16 pairs: a piece is the rest rounded to bf16, the next rest is exact, and the
-// third piece holds what is left exactly.
+// third piece holds what is left: exactly for magnitudes from 2^-110 up to the largest fp32 value, below that
+// to the last bit of bf16's subnormals (2^-133).  The pieces of an infinity or a NaN add up to it again.
 __device__ __forceinline__ void split_pair(float a, float b, uint32_t& p1, uint32_t& p2, uint32_t& p3) {
-  p1 = bf16_pair(a, b);
+  p1 = bf16_pair_sat(a, b);
   a -= __uint_as_float(p1 << 16);
   b -= __uint_as_float(p1 & 0xFFFF0000u);
-  p2 = bf16_pair(a, b);
+  p2 = bf16_pair_sat(a, b);
   a -= __uint_as_float(p2 << 16);
   b -= __uint_as_float(p2 & 0xFFFF0000u);
   p3 = bf16_pair(a, b);
@@ -1684,7 +1691,8 @@ __global__ void __launch_bounds__(128) dense_weights_kernel(const DeviceLayer L)
       } else {
         float rest = v;
         for (int p = 0; p < 3; ++p) {
-          const uint32_t piece = (__float_as_uint(rest) + 0x8000u) & 0xFFFF0000u;
+          uint32_t piece = (__float_as_uint(rest) + 0x8000u) & 0xFFFF0000u;
+          if ((piece & 0x7F800000u) == 0x7F800000u) piece -= 0x10000u;    // (packed weights are finite)
           d[(size_t)p * L.dense_rows * 8] = (unsigned short)(piece >> 16);
           rest -= __uint_as_float(piece);
         }
