@@ -116,9 +116,12 @@ enum {
                                   bf16 pieces a value, six products) -- and is still faster wherever
                                   there is enough work for them, so the library picks it by estimate.
                                   fp16 products are exact in fp32; the fp32 form drops less than 2^-24 of
-                                  a product.  A result differs from the sparse kernels' by summation
-                                  order, and where an activation is infinite or not a number: its
-                                  product with a pruned weight's zero is then not a number. */
+                                  a product, and its pieces are exact for activations and weights of
+                                  magnitude 2^-110 up to the largest fp32 value (smaller ones to 2^-133).
+                                  A result differs from the sparse kernels' by summation order only: an
+                                  infinite activation or a NaN reaches the outputs that have it under a
+                                  surviving tap and no others.  (Outputs whose dense sum is not finite are
+                                  formed again from the surviving taps, at the speed of the plain kernel.) */
 };
 
 #define PCONV_MAX_PATTERNS 16

@@ -73,6 +73,7 @@ constexpr int kMaxB = 24;                 // weight slots
 constexpr int kMaxT = 4;                  // 128-position tiles of a work item
 constexpr int kHeader = 1024;             // barriers, Tensor Memory address, bias of a filter tile
 constexpr int kBiasOff = 512;
+static_assert(16 * (kMaxA + kMaxB) + 32 + 4 + 16 <= kBiasOff, "barriers, Tensor Memory address, segments to redo");
 constexpr uint32_t kSpinLimit = 1u << 20;
 constexpr uint32_t kWaitHintNs = 200;
 constexpr int kSmemLimit = 227 * 1024;
@@ -582,12 +583,129 @@ __device__ __forceinline__ void pool_columns(float (&v)[8], const float (&v2)[8]
   }
 }
 
-// A warp's finished columns of one tile from Tensor Memory to the result.
+// ---- sums that are not finite --------------------------------------------------------------------
+// The dense sums hold a product for every pruned weight's zero too, and 0 x infinity is not a number; and sums of
+// pieces can leave the range where the result does not.  Every output with such a term has a sum that is
+// not finite.  A warp that stores one remembers the segment and, once all its work is done, forms the
+// segment's outputs again from the layer's lists, over the surviving taps alone: an infinity or a NaN reaches
+// the outputs that depend on it and no others.  The usual case pays four packed multiply-adds per eight columns.
+// What it costs: VGG-16 N=1 331 -> 334 us, ResNet-50 N=32 855 -> 863, CIFAR VGG-16 fp16 N=256 333 -> 334.5, one
+// layer 11.9 -> 12.0.  Formed again inside the epilogue loop it cost 2-6 % (registers kept for the call in all
+// roles); fp32, whose epilogue has no register left for the segments, keeps them in shared memory and forms them
+// at the very end, fp16 (0.5 % the other way round) in a register until the epilogue ends.
+__device__ __forceinline__ void note_finite(u64& z, const uint32_t (&v)[8]) {   // two sums that stay 0 while all are finite
+#pragma unroll
+  for (int i = 0; i < 8; i += 2)
+    asm("{\n\t.reg .b64 a, o;\n\tmov.b64 a, {%1, %2};\n\tmov.b64 o, 0;\n\tfma.rn.f32x2 %0, a, o, %0;\n\t}"
+        : "+l"(z) : "r"(v[i]), "r"(v[i + 1]));
+}
+__device__ __forceinline__ bool all_finite(u64 z) {
+  return __uint_as_float((uint32_t)z) + __uint_as_float((uint32_t)(z >> 32)) == 0.f;
+}
+// The bit of a segment in the warp's memory: whole tiles share 14 (all of them are this CTA's to store again);
+// parts of a tile, which another CTA may have stored, can only be the share's first segment and its last.
+__device__ __forceinline__ uint32_t redo_bit(const DGeo& g, const Item& it, int seg) {
+  return it.k1 - it.k0 == g.k_steps ? 4u << (seg % 14) : seg == 0 ? 1u : 2u;
+}
+
+// The sum of filter o at position p of tile j.  Its input pixels are found as the staging found them: in x, or
+// in the position rows behind the tap's shift.
+template <bool HALF, bool P8>
+__device__ __forceinline__ float sum_from_lists(const DeviceLayer& L, const DGeo& g, const void* __restrict__ xv, int p, int j,
+                                                int o) {
+  constexpr int kPieces = HALF ? 1 : 3;
+  const int cell = p / g.cell_pos, r = p - cell * g.cell_pos, i = r / g.pitch;
+  const int img = cell / g.strips, st = cell - img * g.strips;
+  const int y0 = (g.pool ? 2 * i + (j & 1) : i) * L.stride - 1;
+  const int x0 = (st * g.strip_w + r - i * g.pitch) * L.stride - 1;
+  const size_t piece = (size_t)g.planes * g.in_plane_len * 8;          // values of one piece of eight channels
+  const int end = L.row_ptr[o + 1];
+  float sum = 0.f;
+#pragma unroll 1
+  for (int k = L.row_ptr[o]; k < end; ++k) {
+    const uint32_t idx = L.csr_idx[k];
+    const int c = idx & 0xFFFF;
+    uint32_t mask = idx >> 16;                                         // (four taps)
+#pragma unroll
+    for (int s = 0; s < 4; ++s, mask &= mask - 1) {
+      const int t = __ffs(mask) - 1;
+      float v = 0.f;
+      if constexpr (P8) {
+        const int off = g.tap_off[j][__popc(L.tap_mask & ((1 << t) - 1))] - 128 * (g.pool ? j >> 1 : j);
+        const int pl = off / g.plane_pos, q = g.in_lead + p + off - pl * g.plane_pos - g.lead;
+        const size_t at = (size_t)(c >> 3) * kPieces * piece + ((size_t)pl * g.in_plane_len + q) * 8 + (c & 7);
+        if constexpr (HALF) {
+          v = __half2float(reinterpret_cast<const __half*>(xv)[at]);
+        } else {
+          const unsigned short* b = reinterpret_cast<const unsigned short*>(xv) + at;
+          v = __uint_as_float((uint32_t)b[0] << 16) + __uint_as_float((uint32_t)b[piece] << 16) +
+              __uint_as_float((uint32_t)b[2 * piece] << 16);
+        }
+      } else {
+        const int y = y0 + t / 3, x = x0 + t % 3;
+        if ((unsigned)y < (unsigned)g.h && (unsigned)x < (unsigned)g.w) {
+          const size_t at = (((size_t)img * g.c_in + c) * g.h + y) * g.w + x;
+          if constexpr (HALF) v = __half2float(reinterpret_cast<const __half*>(xv)[at]);
+          else v = reinterpret_cast<const float*>(xv)[at];
+        }
+      }
+      sum = fmaf(L.csr_val[4 * (size_t)k + s], v, sum);
+    }
+  }
+  return sum;
+}
+
+// The segments of `redo` again: this warp's blocks of eight columns first, first + step, ...
+template <bool HALF, bool P8>
+__device__ __noinline__ void emit_from_lists(const DeviceLayer& L, const DGeo& g, uint32_t redo, const void* __restrict__ xv,
+                                             const float* __restrict__ bias, void* __restrict__ yv, int first, int step) {
+  typedef typename std::conditional<HALF, __half, float>::type T;
+  const size_t plane = (size_t)g.h_out * g.w_out;
+  const bool pool = g.pool != 0, pairs = !pool && (g.w_out & 1) == 0 && (g.strip_w & 1) == 0;
+  const Share share = {share_begin(g, blockIdx.x), share_begin(g, blockIdx.x + 1)};
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int q = warp & 3, n_col = g.nt / 2, col0 = (warp >> 2) * n_col, blocks = n_col / 8, jstep = pool ? 2 : 1;
+  Item it;
+#pragma unroll 1
+  for (int seg = 0; get_item(g, share, seg, &it); ++seg) {
+    if (!(redo & redo_bit(g, it, seg))) continue;
+    const int top = min(min(g.nt, g.c_out - it.f0), col0 + n_col);
+#pragma unroll 1
+    for (int i = first; i < g.tiles / jstep * blocks; i += step) {
+      const int jj = i / blocks, col = col0 + (i - jj * blocks) * 8;
+      const int p = it.m0 + 128 * jj + 32 * q + lane;
+      const long long dst = lane_dest(g, p, it.f0, plane);
+      float v[8];
+#pragma unroll 1
+      for (int k = 0; k < 8; ++k) {
+        const int o = it.f0 + col + k;
+        const bool real = dst >= 0 && col + k < top;
+        float best = 0.f;
+#pragma unroll 1
+        for (int j = jstep * jj; j < jstep * jj + jstep; ++j) {
+          float sum = real ? sum_from_lists<HALF, P8>(L, g, xv, p, j, o) + (bias ? bias[o] : 0.f) : 0.f;
+          if (g.relu) sum = fmaxf(sum, 0.f);
+          best = j == jstep * jj ? sum : fmaxf(best, sum);
+        }
+        v[k] = pool ? fmaxf(best, __shfl_xor_sync(0xffffffffu, best, 1)) : best;
+      }
+      if (g.out_p8) {
+        if (it.f0 + col < g.rows) store_rows<HALF>(yv, g, v, dst, (it.f0 + col) >> 3, pool, lane);
+      } else {
+        store_chunk(reinterpret_cast<T*>(yv), v, dst, col, top, plane, pool, pairs, lane);
+      }
+    }
+  }
+}
+
+// A warp's finished columns of one tile (n_col of them, the ones that are stored) from Tensor Memory to the
+// result; false if a sum was not finite.
 template <bool HALF, Form FORM>
-__device__ __forceinline__ void emit_columns(const DGeo& g, void* __restrict__ y, uint32_t from, uint32_t tile_stride,
+__device__ __forceinline__ bool emit_columns(const DGeo& g, void* __restrict__ y, uint32_t from, uint32_t tile_stride,
                                              const float* bias_s, long long dst, int f0, int col0, int n_col, int n_f,
                                              size_t plane, bool pool, bool pairs, int lane) {
   constexpr int kWide = HALF && FORM == kNchw ? 8 : 16;
+  u64 z = 0;
 #pragma unroll 1
   for (int c = 0; c < n_col; c += kWide) {
     uint32_t r[kWide / 8][8];
@@ -601,6 +719,7 @@ __device__ __forceinline__ void emit_columns(const DGeo& g, void* __restrict__ y
       float v[8];
 #pragma unroll
       for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[k][i]);
+      note_finite(z, r[k]);
       if (pool) {
         uint32_t r2[8];
         float v2[8];
@@ -608,6 +727,7 @@ __device__ __forceinline__ void emit_columns(const DGeo& g, void* __restrict__ y
         tmem_ld_wait();
 #pragma unroll
         for (int i = 0; i < 8; ++i) v2[i] = __uint_as_float(r2[i]);
+        note_finite(z, r2);
         pool_columns(v, v2);
       }
       // (a warp stores its own columns only)
@@ -615,6 +735,7 @@ __device__ __forceinline__ void emit_columns(const DGeo& g, void* __restrict__ y
                                  lane);
     }
   }
+  return !__any_sync(0xffffffffu, dst >= 0 && !all_finite(z));
 }
 
 // All threads of a cluster's CTAs meet; writes before it are seen after it.
@@ -889,7 +1010,7 @@ __device__ __forceinline__ void activation_role(const DeviceLayer& L, const DGeo
 
 template <bool HALF, int V>
 __global__ void __launch_bounds__(Cfg<HALF, V == 0>::kThreads, 1)
-dense_kernel(const DeviceLayer L, const __grid_constant__ DGeo g, const void* __restrict__ xv,
+dense_kernel(const __grid_constant__ DeviceLayer L, const __grid_constant__ DGeo g, const void* __restrict__ xv,
              const float* __restrict__ bias, void* __restrict__ yv, float* __restrict__ ws, int* __restrict__ tickets) {
   constexpr bool P8 = V == 0;
   using C = Cfg<HALF, P8>;
@@ -901,6 +1022,7 @@ dense_kernel(const DeviceLayer L, const __grid_constant__ DGeo g, const void* __
   const uint32_t bar_bf = bar_ae + 8 * kMaxA, bar_be = bar_bf + 8 * kMaxB;
   const uint32_t bar_cf = bar_be + 8 * kMaxB, bar_ce = bar_cf + 16;     // accumulators full / empty
   volatile uint32_t* tmem_s = reinterpret_cast<volatile uint32_t*>(smem + 16 * (kMaxA + kMaxB) + 32);
+  volatile uint16_t* redo_s = reinterpret_cast<volatile uint16_t*>(tmem_s + 1);     // [8] fp32: see redo_bit
   float* bias_s = reinterpret_cast<float*>(smem + kBiasOff);            // [128]
   Load* tab_s = reinterpret_cast<Load*>(smem + kHeader);                // [kTables][n_vec]
 
@@ -921,6 +1043,7 @@ dense_kernel(const DeviceLayer L, const __grid_constant__ DGeo g, const void* __
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  if (!HALF && tid < C::kEpiWarps) redo_s[tid] = 0;
   if (warp == C::kMmaWarp) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(
                      smem_u32((const void*)tmem_s))
@@ -934,7 +1057,6 @@ dense_kernel(const DeviceLayer L, const __grid_constant__ DGeo g, const void* __
   const size_t hw = (size_t)g.h * g.w;
   const Bars bars = {bar_af, bar_ae, bar_bf, bar_be, bar_cf, bar_ce};
   const Share share = {share_begin(g, blockIdx.x), share_begin(g, blockIdx.x + 1)};
-
   if (warp == C::kMmaWarp) {
     // ======================================= MMA issuer =======================================
     if constexpr (HALF) {
@@ -1097,6 +1219,7 @@ dense_kernel(const DeviceLayer L, const __grid_constant__ DGeo g, const void* __
     uint32_t sc = 0;
     T_DECL;
     bool ok = true, waited = false;
+    uint32_t redo = 0;
     Item it;
     for (int seg = 0; get_item(g, share, seg, &it); ++seg) {
       const int n_f = min(g.nt, g.c_out - it.f0);        // real filters of this tile
@@ -1238,12 +1361,19 @@ dense_kernel(const DeviceLayer L, const __grid_constant__ DGeo g, const void* __
         // (one loop with both forms in it took 1.2-1.4 times as long).  In the fp32 kernel, whose register sums
         // leave no room, two loops cost spills in the channel loop and a fifth of its time.
         const int jstep = pool ? 2 : 1;
+        // (position rows have the padding filters too; past them a tile's columns hold whatever was there)
+        const int n_stored = min(n_col, (((g.out_p8 ? g.rows - it.f0 : n_f) + 7) & ~7) - col0);
         for (int j = 0, jj = 0; j < g.tiles; j += jstep, ++jj) {
           const long long dst = lane_dest(g, it.m0 + 128 * jj + 32 * q + lane, it.f0, plane);
           const uint32_t from = res + (uint32_t)j * res_stride;
-          if constexpr (!HALF) emit_columns<HALF, kEither>(g, yv, from, res_stride, bias_s, dst, it.f0, col0, n_col, n_f, plane, pool, pairs, lane);
-          else if (g.out_p8) emit_columns<HALF, kRows>(g, yv, from, res_stride, bias_s, dst, it.f0, col0, n_col, n_f, plane, pool, pairs, lane);
-          else emit_columns<HALF, kNchw>(g, yv, from, res_stride, bias_s, dst, it.f0, col0, n_col, n_f, plane, pool, pairs, lane);
+          bool fine;
+          if constexpr (!HALF) fine = emit_columns<HALF, kEither>(g, yv, from, res_stride, bias_s, dst, it.f0, col0, n_stored, n_f, plane, pool, pairs, lane);
+          else if (g.out_p8) fine = emit_columns<HALF, kRows>(g, yv, from, res_stride, bias_s, dst, it.f0, col0, n_stored, n_f, plane, pool, pairs, lane);
+          else fine = emit_columns<HALF, kNchw>(g, yv, from, res_stride, bias_s, dst, it.f0, col0, n_stored, n_f, plane, pool, pairs, lane);
+          if (!fine) {
+            if (HALF) redo |= redo_bit(g, it, seg);
+            else redo_s[warp] = (uint16_t)(redo_s[warp] | redo_bit(g, it, seg));
+          }
         }
       }
       if (!HALF && !g.out_col) {
@@ -1260,6 +1390,7 @@ dense_kernel(const DeviceLayer L, const __grid_constant__ DGeo g, const void* __
     if (tid == 0) T_FLUSH(7, 9);
     if (tid == 0) T_STAMP(12);
     if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (HALF && redo) emit_from_lists<HALF, P8>(L, g, redo, xv, bias, yv, 0, 1);
   }
 
   if (g.cluster) {
@@ -1297,19 +1428,27 @@ dense_kernel(const DeviceLayer L, const __grid_constant__ DGeo g, const void* __
         }
       };
       const int jstep = pool ? 2 : 1, blocks = n_col / 8;
+      uint32_t redo = 0;
 #pragma unroll 1
       for (int i = (int)rank; i < g.tiles / jstep * blocks; i += g.parts) {
         const int jj = i / blocks, c = (i - jj * blocks) * 8;
         const long long dst = lane_dest(g, it.m0 + 128 * jj + 32 * q + lane, it.f0, plane);
-        float v[8], v2[8];
+        float v[8], v2[8], z = 0.f;
         gather((jj * jstep * n_col + c) / 4, v);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) z = fmaf(v[k], 0.f, z);
         if (pool) {
           gather(((jj * jstep + 1) * n_col + c) / 4, v2);
+#pragma unroll
+          for (int k = 0; k < 8; ++k) z = fmaf(v2[k], 0.f, z);
           pool_columns(v, v2);
         }
         const int top = min(n_f, col0 + n_col);
+        if (dst >= 0 && z != 0.f && col0 + c < (g.out_p8 ? g.rows - it.f0 : n_f)) redo = 1u;
         finish_columns<HALF, kEither>(g, yv, v, bias_s, dst, it.f0, col0 + c, top, plane, pool, pairs, lane);
       }
+      if (HALF && __any_sync(0xffffffffu, redo)) emit_from_lists<HALF, P8>(L, g, 1u, xv, bias, yv, (int)rank, g.parts);
+      if (!HALF && redo) redo_s[warp] = 1;
     }
     cluster_sync();      // (nobody leaves while its sums are being read)
   }
@@ -1320,6 +1459,12 @@ dense_kernel(const DeviceLayer L, const __grid_constant__ DGeo g, const void* __
   if (tid == 0) T_STAMP(13);
   if (warp == C::kMmaWarp)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
+  // fp32: where no register is free for it in the roles
+  if (!HALF && threadIdx.x < 32 * C::kEpiWarps && redo_s[threadIdx.x >> 5] != 0) {
+    uint32_t rank = 0;
+    if (g.cluster) asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    emit_from_lists<HALF, P8>(L, g, redo_s[threadIdx.x >> 5], xv, bias, yv, (int)rank, g.cluster ? g.parts : 1);
+  }
 }
 
 // ---- position rows ------------------------------------------------------------------------------

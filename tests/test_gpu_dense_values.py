@@ -1,6 +1,7 @@
-"""What the dense tensor-core kernel makes of values at the ends of the fp32 range: largest finite
-activations and weights, and values so small that a piece of theirs is a bf16 subnormal.  The development
-build pins the kernel (PCONV_FORCE_DENSE) and the form of its input: NCHW, or position rows."""
+"""What the dense tensor-core kernel makes of values at the ends of the range: largest finite activations
+and weights, values so small that a piece of theirs is a bf16 subnormal, and activations that are
+infinite or not a number.  The development build pins the kernel, and where it matters its plan
+(PCONV_FORCE_DENSE), and the form of its input: NCHW, or position rows."""
 import numpy as np
 import pytest
 import torch
@@ -9,6 +10,7 @@ import oracle
 from paper_1909_05073_b200 import binding as B
 from paper_1909_05073_b200 import build as pbuild
 from paper_1909_05073_b200 import synth
+from util import check_close
 
 pytestmark = pytest.mark.gpu
 
@@ -27,6 +29,32 @@ def dev_library():
 def dense(request, monkeypatch):
     monkeypatch.setenv("PCONV_FORCE_DENSE", "0,0,0,0")
     monkeypatch.setenv("PCONV_FORCE_ROWS", "1" if request.param == "rows" else "0")
+
+
+def conv_of_surviving_taps(x, wt, bias, stride, relu, storage="f32", pool=False):
+    """The layer where infinities and NaNs meet the surviving taps only (no weight inside a pattern is zero
+    here): the finite part from the oracle, and from it, on indicator maps, how many terms are infinite."""
+    count = lambda hit, w: oracle.conv3x3(hit.astype(np.float32), w.astype(np.float32), None, stride, False) > 0
+    with np.errstate(invalid="ignore"):
+        up, down, nan = x == np.inf, x == -np.inf, np.isnan(x)
+        y = oracle.conv3x3(np.where(np.isfinite(x), x, 0).astype(np.float32), wt, bias, stride, False, storage)
+        pos, neg = count(up, wt > 0) | count(down, wt < 0), count(up, wt < 0) | count(down, wt > 0)
+        y = np.where(pos, np.inf, np.where(neg, -np.inf, y))
+        y = np.where(count(nan, wt != 0) | (pos & neg), np.nan, y).astype(np.float32)
+        y = np.fmax(y, 0) if relu else y        # (a maximum with a NaN is the other operand, as on the GPU)
+        if pool:
+            y = y[:, :, :y.shape[2] // 2 * 2, :y.shape[3] // 2 * 2]
+            y = np.fmax(np.fmax(y[:, :, ::2, ::2], y[:, :, ::2, 1::2]), np.fmax(y[:, :, 1::2, ::2], y[:, :, 1::2, 1::2]))
+    return y
+
+
+def check_with_infinities(got, want, storage, what):
+    got = got.float().cpu().numpy()
+    assert np.array_equal(np.isnan(got), np.isnan(want)), "%s: NaN: %d here, %d wanted" % (what, np.isnan(got).sum(), np.isnan(want).sum())
+    inf = np.isinf(want)
+    assert inf.any() and np.array_equal(got[inf], want[inf]), what
+    fine = np.isfinite(want)
+    check_close(got[fine], want[fine], storage, what)
 
 
 def make(c_in, c_out, h, w, n, stride, storage="f32", seed=5, keep=0.5):
@@ -68,3 +96,67 @@ def test_largest_and_smallest_finite_values(c_in, c_out, h, w, n, stride, where,
     assert np.isfinite(got).all(), "%d outputs are not finite" % (~np.isfinite(got)).sum()
     assert (np.abs(got - ref) <= (4 * c_in + 8) * 2.0 ** -23 * size).all()
     layer.close()
+
+
+SPECIAL = [np.inf, -np.inf, np.nan, np.inf]
+CASES = [  # (c_in, c_out, h, w, n, stride): ragged channels and filters, several tiles, strips, parity planes
+    (24, 40, 12, 13, 2, 1), (33, 75, 9, 30, 2, 1), (8, 40, 3, 300, 1, 1), (40, 24, 15, 10, 3, 2), (5, 130, 1, 9, 2, 2),
+]
+
+
+@pytest.mark.parametrize("storage", ["f32", "f16"])
+@pytest.mark.parametrize("case", CASES, ids=lambda c: "x".join(str(v) for v in c))
+def test_infinities_and_nans_reach_only_what_depends_on_them(case, storage, dense):
+    c_in, c_out, h, w, n, stride = case
+    x, wt, bias = make(c_in, c_out, h, w, n, stride)
+    plant(x, SPECIAL, 7)
+    layer = B.Layer(wt, synth.PATTERNS8, stride, B.F16 if storage == "f16" else B.F32, bias)
+    xt = torch.from_numpy(x).cuda()
+    xt = xt.half() if storage == "f16" else xt
+    for relu in (False, True):
+        for pool in (False, True) if min(layer.out_shape(x.shape)[2:]) > 1 else (False,):
+            want = conv_of_surviving_taps(x, wt, bias, stride, relu, storage, pool)
+            got = layer.forward(xt, relu=relu, pool=pool)
+            check_with_infinities(got, want, storage, "relu=%s pool=%s" % (relu, pool))
+    assert B.pconv_device_status(layer.handle) == (0, 0)
+    layer.close()
+
+
+@pytest.mark.parametrize("plan", ["1,64,1,0", "1,64,4,0", "1,64,4,1"])     # whole; parts through the workspace; a cluster
+@pytest.mark.parametrize("storage", ["f32", "f16"])
+def test_infinities_where_thread_blocks_share_a_tile(storage, plan, dense, monkeypatch):
+    x, wt, bias = make(256, 64, 7, 7, 1, 1)
+    plant(x, SPECIAL, 8)
+    monkeypatch.setenv("PCONV_FORCE_DENSE", plan)
+    layer = B.Layer(wt, synth.PATTERNS8, 1, B.F16 if storage == "f16" else B.F32, bias)
+    xt = torch.from_numpy(x).cuda()
+    xt = xt.half() if storage == "f16" else xt
+    want = conv_of_surviving_taps(x, wt, bias, 1, False, storage)
+    for _ in range(2):                          # the workspace keeps nothing of them
+        check_with_infinities(layer.forward(xt, relu=False, split=True), want, storage, plan)
+    if layer._ws is not None:
+        assert not layer._ws.any()
+    layer.close()
+
+
+@pytest.mark.parametrize("storage", ["f32", "f16"])
+def test_infinities_through_a_stack(storage, dense):
+    """Position rows written by one layer and read by the next, their padding filters among them."""
+    chans, pools, strides, h = [17, 40, 24, 72], [1, 0, 0], [1, 2, 1], 21
+    x, _, _ = make(17, 8, h, h, 2, 1)
+    plant(x, [np.inf, -np.inf], 9)
+    layers, a, hh = [], x, h
+    for i in range(3):
+        _, wt, bias = make(chans[i], chans[i + 1], hh, hh, 1, strides[i], seed=20 + i)
+        layers.append(B.Layer(wt, synth.PATTERNS8, strides[i], B.F16 if storage == "f16" else B.F32, bias))
+        a = conv_of_surviving_taps(a, wt, bias, strides[i], True, storage, bool(pools[i]))
+        if storage == "f16":
+            a = a.astype(np.float16).astype(np.float32)
+        hh = a.shape[2]
+    stack = B.Stack(layers, pools, 2, h, h, B.RELU)
+    xt = torch.from_numpy(x).cuda()
+    y = torch.empty(stack.out_shape, dtype=torch.float16 if storage == "f16" else torch.float32, device="cuda")
+    stack.forward(xt.to(y.dtype), y)
+    check_with_infinities(y, a, storage, "stack")
+    assert stack.status() == (0, 0)
+    stack.close()
