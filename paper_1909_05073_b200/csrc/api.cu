@@ -207,12 +207,14 @@ static pconv_status forward_impl(const pconv_handle* h, const void* x, const flo
   // rows staged in the caller's scratch memory if there is enough of it
   void* dense_ws = repro ? nullptr : ws;
   const size_t dense_ws_bytes = dense_ws ? ws_bytes : 0;
-  const size_t rows = scratch ? dense_rows_bytes(L, n, h_in, w_in, pool) : 0;
-  const DensePath path = dense_path(L, n, h_in, w_in, pool, rows > 0 && rows <= scratch_bytes ? kRowsStaged : kNoRows,
-                                    dense_ws_bytes);
-  const bool staged = path == kFromRows;
-  const bool dense = sel == 0 && rmode == 0 && !cluster &&
-                     (path != kNotDense || (!pool && batch_on_tensor_cores(L, n, h_in, w_in)));
+  bool dense = false, staged = false;
+  if (sel == 0 && rmode == 0 && !cluster) {
+    const size_t rows = scratch ? dense_rows_bytes(L, n, h_in, w_in, pool) : 0;
+    const DensePath path = dense_path(L, n, h_in, w_in, pool, rows > 0 && rows <= scratch_bytes ? kRowsStaged : kNoRows,
+                                      dense_ws_bytes);
+    staged = path == kFromRows;
+    dense = path != kNotDense || (!pool && batch_on_tensor_cores(L, n, h_in, w_in));
+  }
   if (pool && !dense && (sel == PCONV_KERNEL_SIMPLE || !tiled_supported(L, n, h_in, w_in)))
     return PCONV_ERR_UNSUPPORTED;  // the plain kernel does not fuse the pool
   if (dense || sel == PCONV_KERNEL_TENSOR) {
@@ -336,6 +338,8 @@ extern "C" pconv_status pconv_dev_withhold(int chunk, unsigned spin_limit) {
   }
   return PCONV_OK;
 }
+
+extern "C" long long pconv_dev_dense_plans(void) { return pconv::dense_plans_made(); }
 
 extern "C" pconv_status pconv_dev_clear_status(const pconv_handle* h) {
   if (!h) return PCONV_ERR_NULL;

@@ -1705,6 +1705,9 @@ double dense_cycles(const DGeo& g, bool half) {
 }
 
 int max_clusters(bool half, int parts);   // below: needs the kernels
+#ifdef PCONV_DEV
+std::atomic<long long> g_plans_made{0};
+#endif
 
 // The geometry of a launch: the cheapest by the estimate.  ws_bytes: workspace the caller has.
 bool dense_plan(const DeviceLayer& L, int n, int h, int w, bool pool, bool p8, size_t ws_bytes, DGeo* out, double* cycles) {
@@ -1714,6 +1717,7 @@ bool dense_plan(const DeviceLayer& L, int n, int h, int w, bool pool, bool p8, s
   bool found = false;
   double best = 0.0;
 #ifdef PCONV_DEV
+  ++g_plans_made;
   int force[4] = {0, 0, 0, 0};
   if (const char* e = getenv("PCONV_FORCE_DENSE")) sscanf(e, "%d,%d,%d,%d", &force[0], &force[1], &force[2], &force[3]);
 #endif
@@ -2034,6 +2038,8 @@ DensePath dense_path(const DeviceLayer& L, int n, int h, int w, bool pool, RowsF
 }
 
 #ifdef PCONV_DEV
+long long dense_plans_made() { return g_plans_made.load(); }
+
 cudaError_t dense_set_withhold(int step, unsigned spin_limit) {
   const unsigned limit = step >= 0 ? spin_limit : kSpinLimit;
   cudaError_t e = cudaMemcpyToSymbol(g_withhold_step, &step, sizeof(step));

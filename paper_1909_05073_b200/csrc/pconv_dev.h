@@ -32,6 +32,10 @@ pconv_status pconv_trace_read(const pconv_handle* h, unsigned long long* words_h
  * restores the normal limit.  Synchronises the device. */
 pconv_status pconv_dev_withhold(int chunk, unsigned spin_limit);
 
+/* Launch plans of the dense tensor-core kernel worked out by this process so far (a call that finds its
+ * plan already made adds none). */
+long long pconv_dev_dense_plans(void);
+
 /* Clears the handle's sticky status word (pconv_device_status reports PCONV_OK again until the
  * next abandoned wait).  Synchronises the device. */
 pconv_status pconv_dev_clear_status(const pconv_handle* h);

@@ -164,6 +164,7 @@ bool tiled_plan(const DeviceLayer& L, int n, int h, int w, bool generic_taps, bo
 #ifdef PCONV_DEV
 cudaError_t dev_set_withhold(int chunk, unsigned spin_limit);     // see pconv_dev.h
 cudaError_t dense_set_withhold(int step, unsigned spin_limit);
+long long dense_plans_made();
 #endif
 // chains: several consecutive layers of a stack in one persistent launch (kernels_tiled.cu)
 bool chain_layer_ok(const DeviceLayer& L, int n, int h, int w, bool pool, long long* ctas);
