@@ -59,8 +59,8 @@ static int rows_mode(unsigned flags) {
 // the case in which a default forward is, without any estimate, the pinned tensor-core kernel.  The
 // zero-inserted contraction at a fifth of the tensor peak must be cheaper than the surviving
 // multiply-adds at a fifth of the FP32 peak.
-static bool batch_on_tensor_cores(const pconv::DeviceLayer& L, int n, int h, int w) {
-  if (L.storage != PCONV_F16 || L.stride != 1 || !dense_supported(L, n, h, w, false)) return false;
+static bool batch_on_tensor_cores(const pconv::DeviceLayer& L, int n, int h, int w, size_t ws_bytes) {
+  if (L.storage != PCONV_F16 || L.stride != 1 || !dense_supported(L, n, h, w, false, ws_bytes)) return false;
   const double tiles = (double)n * (h + 1) * (w + 1) / 128.0 * ((L.dense_rows + 127) / 128);
   if (tiles < device_sm_count() / 4) return false;
   const double dense = 2.0 * 9.0 * (16.0 * ((L.c_in + 15) / 16)) * L.dense_rows, sparse = 8.0 * (double)L.n_kept;
@@ -101,7 +101,7 @@ extern "C" pconv_status pconv_plan(const pconv_handle* h, int n, int h_in, int w
   if (!tiled_plan(h->d, n, h_in, w_in, (flags & PCONV_KERNEL_GENERIC_TAPS) != 0, with_workspace != 0,
                   rows_mode(flags), plan))
     return PCONV_ERR_UNSUPPORTED;
-  plan->tensor_path = batch_on_tensor_cores(h->d, n, h_in, w_in) ? 1 : 0;
+  plan->tensor_path = batch_on_tensor_cores(h->d, n, h_in, w_in, 0) ? 1 : 0;
   return PCONV_OK;
 }
 
@@ -154,7 +154,7 @@ extern "C" pconv_status pconv_scratch_bytes(const pconv_handle* h, int n, int h_
   if (n < 0 || h_in <= 0 || w_in <= 0) return PCONV_ERR_SHAPE;
   *bytes = 0;
   for (int pool = 0; n > 0 && pool < 2; ++pool)
-    *bytes = std::max(*bytes, dense_rows_bytes(h->d, n, h_in, w_in, pool != 0));
+    *bytes = std::max(*bytes, dense_rows_bytes(h->d, n, h_in, w_in, pool != 0, pconv::kMaxSplitBytes));
   return PCONV_OK;
 }
 
@@ -209,16 +209,16 @@ static pconv_status forward_impl(const pconv_handle* h, const void* x, const flo
   const size_t dense_ws_bytes = dense_ws ? ws_bytes : 0;
   bool dense = false, staged = false;
   if (sel == 0 && rmode == 0 && !cluster) {
-    const size_t rows = scratch ? dense_rows_bytes(L, n, h_in, w_in, pool) : 0;
+    const size_t rows = scratch ? dense_rows_bytes(L, n, h_in, w_in, pool, dense_ws_bytes) : 0;
     const DensePath path = dense_path(L, n, h_in, w_in, pool, rows > 0 && rows <= scratch_bytes ? kRowsStaged : kNoRows,
                                       dense_ws_bytes);
     staged = path == kFromRows;
-    dense = path != kNotDense || (!pool && batch_on_tensor_cores(L, n, h_in, w_in));
+    dense = path != kNotDense || (!pool && batch_on_tensor_cores(L, n, h_in, w_in, dense_ws_bytes));
   }
   if (pool && !dense && (sel == PCONV_KERNEL_SIMPLE || !tiled_supported(L, n, h_in, w_in)))
     return PCONV_ERR_UNSUPPORTED;  // the plain kernel does not fuse the pool
   if (dense || sel == PCONV_KERNEL_TENSOR) {
-    if (!dense && (pool || L.storage != PCONV_F16 || L.stride != 1 || !dense_supported(L, n, h_in, w_in, false)))
+    if (!dense && (pool || L.storage != PCONV_F16 || L.stride != 1 || !dense_supported(L, n, h_in, w_in, false, dense_ws_bytes)))
       return PCONV_ERR_UNSUPPORTED;
     e = staged ? launch_stage(L, x, scratch, n, h_in, w_in, pool, stream) : cudaSuccess;
     if (e == cudaSuccess)
@@ -438,7 +438,7 @@ static bool build_chains(pconv_stack* s) {
       hi[i] = ch;
       wi[i] = cw;
       ok[i] = pconv::chain_layer_ok(L, s->n, ch, cw, s->pool[i] != 0, nullptr) &&
-              !batch_on_tensor_cores(L, s->n, ch, cw);
+              !batch_on_tensor_cores(L, s->n, ch, cw, s->ws_bytes);
       ch = (ch - 1) / L.stride + 1;
       cw = (cw - 1) / L.stride + 1;
       if (s->pool[i]) {
@@ -525,12 +525,12 @@ static bool build_rows(pconv_stack* s) {
     for (const pconv_stack::Chain& c : *s->chains) chained = chained || (i >= c.begin && i < c.end);
     const bool pool = s->pool[i] != 0;
     if (!chained) {
-      const size_t bytes = pconv::dense_rows_bytes(L, s->n, ch, cw, pool);
+      const size_t bytes = pconv::dense_rows_bytes(L, s->n, ch, cw, pool, ws_bytes);
       const bool given = bytes > 0 && i > 0 && (*s->path)[i - 1] != pconv::kNotDense;
       (*s->path)[i] = pconv::dense_path(L, s->n, ch, cw, pool,
                                         given ? pconv::kRowsGiven : bytes > 0 ? pconv::kRowsStaged : pconv::kNoRows, ws_bytes);
-      if ((*s->path)[i] == pconv::kNotDense && batch_on_tensor_cores(L, s->n, ch, cw) &&
-          pconv::dense_supported(L, s->n, ch, cw, pool))
+      if ((*s->path)[i] == pconv::kNotDense && batch_on_tensor_cores(L, s->n, ch, cw, ws_bytes) &&
+          pconv::dense_supported(L, s->n, ch, cw, pool, ws_bytes))
         (*s->path)[i] = pconv::kFromNchw;
       if ((*s->path)[i] == pconv::kFromRows) {
         at[i] = total + 1;

@@ -58,7 +58,8 @@
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
-#include <memory>
+#include <cstring>
+#include <mutex>
 #include <type_traits>
 
 #include "pconv_internal.h"
@@ -1771,49 +1772,76 @@ bool dense_plan(const DeviceLayer& L, int n, int h, int w, bool pool, bool p8, s
   return found;
 }
 
-// The plans of recent launches, one small table per thread: planning takes tens of microseconds, a
-// repeated call finds its plan in well under one.
+// The plans of recent launches, one table for the process: planning takes microseconds, a repeated call finds its
+// plan in a tenth of one.  A plan is kept by all that it depends on, which is a layer's geometry and not the
+// layer (ResNet-50's sixteen 3x3 layers have seven), and for every workspace from the one it needs up to
+// the one it was made for: what was the cheapest of more choices is the cheapest of fewer.
 struct PlanKey {
-  long long layer;
-  size_t ws_bytes;
-  int n, h, w, pool, p8, dev_sms;
+  int c_in, c_out, stride, storage, tap_mask, n, h, w, form, dev;      // form: 2 pool + position rows
+};
+struct Plan {
+  bool found;
+  double cycles;
+  size_t need;                 // workspace
+  int n_tiles, n_ft;
 };
 struct PlanEntry {
   PlanKey key;
-  bool found;
-  double cycles;
+  size_t most;                 // it holds for workspaces from plan.need to this
+  Plan plan;
   DGeo geo;
 };
-// Eight entries a set, the oldest replaced: with one entry a set, a few of the 48 keys of a 16-layer
-// network always met, and each pass planned those again (ResNet-50 N=1: 309 us a pass, now 268).
-const PlanEntry& cached_plan(const DeviceLayer& L, int n, int h, int w, bool pool, bool p8, size_t ws_bytes) {
-  constexpr int kSets = 64, kWays = 8;
-  struct Table {
-    PlanEntry entry[kSets][kWays] = {};             // (layer ids start at 1: a zeroed entry matches nothing)
-    unsigned char next[kSets] = {};
-  };
-  static thread_local std::unique_ptr<Table> table;
-  if (!table) table.reset(new Table);
+constexpr int kPlanSets = 64, kPlanWays = 8;       // (the oldest of a set is replaced)
+struct PlanTable {
+  std::mutex lock;
+  PlanEntry entry[kPlanSets][kPlanWays];           // (zeroed: no key has n = 0)
+  unsigned char next[kPlanSets];
+};
+PlanTable g_plans;
+
+Plan find_plan(const DeviceLayer& L, int n, int h, int w, bool pool, bool p8, size_t ws_bytes, DGeo* geo = nullptr) {
+  if (!L.wdense || n <= 0 || h <= 0 || w <= 0) return Plan{};
   if (ws_bytes > kMaxSplitBytes) ws_bytes = kMaxSplitBytes;
-  const PlanKey k = {L.id, ws_bytes, n, h, w, pool ? 1 : 0, p8 ? 1 : 0, device_sm_count()};
-  unsigned long long hash = (unsigned long long)k.layer * 0x9E3779B97F4A7C15ull;
-  hash = (hash ^ (unsigned)n ^ ((unsigned long long)h << 20) ^ ((unsigned long long)w << 40)) * 0x9E3779B97F4A7C15ull;
-  hash = (hash ^ (ws_bytes << 2) ^ (unsigned)(2 * k.pool + k.p8)) * 0x9E3779B97F4A7C15ull;
-  const int set = (int)((hash >> 40) % kSets);
-  for (PlanEntry& o : table->entry[set])
-    if (o.key.layer == k.layer && o.key.ws_bytes == k.ws_bytes && o.key.n == n && o.key.h == h && o.key.w == w &&
-        o.key.pool == k.pool && o.key.p8 == k.p8 && o.key.dev_sms == k.dev_sms)
-      return o;
-  PlanEntry& e = table->entry[set][table->next[set]++ % kWays];
-  e.found = dense_plan(L, n, h, w, pool, p8, ws_bytes, &e.geo, &e.cycles);
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess) cudaGetLastError();
+  const PlanKey k = {L.c_in, L.c_out, L.stride, L.storage, L.tap_mask, n, h, w, 2 * (int)pool + (int)p8, dev};
+  unsigned long long hash = 0;
+  for (int v : {k.c_in, k.c_out, k.n, k.h, k.w, (k.tap_mask << 8) + (k.form << 4) + (k.stride << 2) + k.storage})
+    hash = (hash ^ (unsigned)v) * 0x9E3779B97F4A7C15ull, hash ^= hash >> 29;
+  const int set = (int)((hash >> 40) % kPlanSets);
 #ifdef PCONV_DEV
-  if (e.found && getenv("PCONV_DENSE_VERBOSE"))
-    fprintf(stderr, "dense %d->%d %dx%d n%d s%d pool%d p8 %d ws%zu: tiles %d nt %d split %d cluster %d grid %d n_tiles %d q %d pitch %d a_stages %d b_slots %d cycles %.0f\n",
-            L.c_in, L.c_out, h, w, n, L.stride, (int)pool, (int)p8, ws_bytes, e.geo.tiles, e.geo.nt, e.geo.split, e.geo.cluster * e.geo.parts, e.geo.grid,
-            e.geo.n_tiles, e.geo.q_tot, e.geo.pitch, e.geo.a_stages, e.geo.b_slots, e.cycles);
+  const bool keep = !getenv("PCONV_FORCE_DENSE");      // (a forced plan is nobody else's)
+#else
+  const bool keep = true;
 #endif
-  e.key = k;
-  return e;
+  if (keep) {
+    std::lock_guard<std::mutex> hold(g_plans.lock);
+    for (const PlanEntry& e : g_plans.entry[set])
+      if (std::memcmp(&e.key, &k, sizeof(k)) == 0 && ws_bytes >= e.plan.need && ws_bytes <= e.most) {
+        if (geo) *geo = e.geo;
+        return e.plan;
+      }
+  }
+  PlanEntry made = {};
+  DGeo& g = made.geo;
+  made.key = k;
+  made.most = ws_bytes;
+  made.plan.found = dense_plan(L, n, h, w, pool, p8, ws_bytes, &g, &made.plan.cycles);
+  if (made.plan.found) made.plan.need = split_bytes(g);
+  made.plan.n_tiles = g.n_tiles;
+  made.plan.n_ft = g.n_ft;
+#ifdef PCONV_DEV
+  if (made.plan.found && getenv("PCONV_DENSE_VERBOSE"))
+    fprintf(stderr, "dense %d->%d %dx%d n%d s%d pool%d p8 %d ws%zu: tiles %d nt %d split %d cluster %d grid %d n_tiles %d q %d pitch %d a_stages %d b_slots %d cycles %.0f\n",
+            L.c_in, L.c_out, h, w, n, L.stride, (int)pool, (int)p8, ws_bytes, g.tiles, g.nt, g.split, g.cluster * g.parts, g.grid,
+            g.n_tiles, g.q_tot, g.pitch, g.a_stages, g.b_slots, made.plan.cycles);
+#endif
+  if (geo) *geo = g;
+  if (keep) {
+    std::lock_guard<std::mutex> hold(g_plans.lock);
+    g_plans.entry[set][g_plans.next[set]++ % kPlanWays] = made;
+  }
+  return made.plan;
 }
 
 // Zero-inserted weights from the per-filter lists: one block per filter, one thread per kernel.  Layout:
@@ -1930,21 +1958,21 @@ cudaError_t dense_build_weights(const DeviceLayer& L, cudaStream_t stream) {
   return cudaGetLastError();
 }
 
-bool dense_supported(const DeviceLayer& L, int n, int h, int w, bool pool) {
-  return cached_plan(L, n, h, w, pool, false, 0).found;
+// (whether there is a plan does not depend on the workspace: whole tiles need none)
+bool dense_supported(const DeviceLayer& L, int n, int h, int w, bool pool, size_t ws_bytes) {
+  return find_plan(L, n, h, w, pool, false, ws_bytes).found;
 }
 
 size_t dense_workspace_bytes(const DeviceLayer& L, int n, int h, int w, size_t most) {
   size_t need = 0;
   for (int v = 0; v < 4; ++v) {
-    const PlanEntry& e = cached_plan(L, n, h, w, v & 1, v & 2, most);
-    if (e.found && split_bytes(e.geo) > need) need = split_bytes(e.geo);
+    need = std::max(need, find_plan(L, n, h, w, v & 1, v & 2, most).need);
   }
   return need;
 }
 
-size_t dense_rows_bytes(const DeviceLayer& L, int n, int h, int w, bool pool) {
-  if (!cached_plan(L, n, h, w, pool, true, 0).found) return 0;
+size_t dense_rows_bytes(const DeviceLayer& L, int n, int h, int w, bool pool, size_t ws_bytes) {
+  if (!find_plan(L, n, h, w, pool, true, ws_bytes).found) return 0;
   return rows_bytes(rows_of(L.c_in, L.stride, n, h, w, pool), L.storage == PCONV_F16);
 }
 
@@ -1972,9 +2000,8 @@ cudaError_t launch_stage(const DeviceLayer& L, const void* x, void* rows, int n,
 cudaError_t launch_dense(const DeviceLayer& L, const void* x, const float* bias, void* y, int n, int h, int w,
                          bool relu, bool pool, bool rows_in, const DenseNext* next, void* ws, size_t ws_bytes,
                          cudaStream_t stream) {
-  const PlanEntry& e = cached_plan(L, n, h, w, pool, rows_in, ws ? ws_bytes : 0);
-  if (!e.found) return cudaErrorInvalidValue;
-  DGeo g = e.geo;
+  DGeo g;
+  if (!find_plan(L, n, h, w, pool, rows_in, ws ? ws_bytes : 0, &g).found) return cudaErrorInvalidValue;
   g.relu = relu ? 1 : 0;
   if (next) {
     const Rows r = rows_of(next->c_in, next->stride, n, g.h_out, g.w_out, next->pool);
@@ -2012,22 +2039,22 @@ DensePath dense_path(const DeviceLayer& L, int n, int h, int w, bool pool, RowsF
   const double macs = 4.0 * (double)L.n_kept * n * ((h - 1) / L.stride + 1) * ((w - 1) / L.stride + 1);
   double best = 1380.0 * (12.0 + 0.008 * L.c_in * L.stride + 2.0 * macs / (0.2 * 74.45e6));
   DensePath path = kNotDense;
-  auto cycles_of = [&](const PlanEntry& e) {
-    return e.cycles + (e.geo.n_tiles <= e.geo.n_ft ? (double)dense_weight_bytes(L) / 1600.0 : 0.0);
+  auto cycles_of = [&](const Plan& e) {
+    return e.cycles + (e.n_tiles <= e.n_ft ? (double)dense_weight_bytes(L) / 1600.0 : 0.0);
   };
 #ifdef PCONV_DEV
   if (getenv("PCONV_FORCE_DENSE")) best = 1e15;
   if (const char* f = getenv("PCONV_FORCE_ROWS")) rows = atoi(f) && rows != kNoRows ? kRowsGiven : kNoRows;
 #endif
   if (rows != kRowsGiven) {
-    const PlanEntry& e = cached_plan(L, n, h, w, pool, false, ws_bytes);
+    const Plan e = find_plan(L, n, h, w, pool, false, ws_bytes);
     if (e.found && cycles_of(e) < best) {
       best = cycles_of(e);
       path = kFromNchw;
     }
   }
   if (rows != kNoRows) {
-    const PlanEntry& e = cached_plan(L, n, h, w, pool, true, ws_bytes);
+    const Plan e = find_plan(L, n, h, w, pool, true, ws_bytes);
     double cycles = cycles_of(e);
     if (e.found && rows == kRowsStaged)
       cycles += 5500.0 + ((double)rows_bytes(rows_of(L.c_in, L.stride, n, h, w, pool), half) +

@@ -2,7 +2,6 @@
 // extraction"), filter grouping balanced by surviving-kernel count and same-pattern ordering
 // inside a block ("filter kernel reorder"), and emission of the compressed value / code streams.
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <memory>
@@ -367,8 +366,6 @@ extern "C" pconv_status pconv_pack(const float* w, int c_out, int c_in, const ui
     d.perm = (const int*)(dev + parts[i_pm].off);
     d.err = (int*)(dev + parts[i_er].off);
     d.wdense = i_wd >= 0 ? dev + parts[i_wd].off : nullptr;
-    static std::atomic<long long> layer_ids{0};
-    d.id = ++layer_ids;
     if (e == cudaSuccess && d.wdense) e = dense_build_weights(d, stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
     if (e != cudaSuccess) {

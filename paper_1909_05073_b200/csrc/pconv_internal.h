@@ -94,7 +94,6 @@ struct DeviceLayer {         // device pointers of one packed layer (passed to k
   const void* wdense;
   int dense_rows;            // filters rounded up to 16
   int tap_mask;              // union of the layer's pattern masks: the taps that are stored
-  long long id;              // unique per packed layer of the process (from 1)
 };
 
 // Status block: one status word, one pad word, kTraceWords 64-bit trace words (written only by
@@ -137,14 +136,15 @@ constexpr size_t kMaxDenseBytes = (size_t)256 << 20;   // layers whose dense wei
 constexpr size_t kMaxSplitBytes = (size_t)24 << 20;    // workspace a split may ask for
 size_t dense_weight_bytes(const DeviceLayer& L);
 cudaError_t dense_build_weights(const DeviceLayer& L, cudaStream_t stream);
-bool dense_supported(const DeviceLayer& L, int n, int h, int w, bool pool);
+bool dense_supported(const DeviceLayer& L, int n, int h, int w, bool pool, size_t ws_bytes);
 enum RowsFrom { kNoRows, kRowsStaged, kRowsGiven };    // position rows: no room, to be staged, already there
 enum DensePath { kNotDense, kFromNchw, kFromRows };
 DensePath dense_path(const DeviceLayer& L, int n, int h, int w, bool pool, RowsFrom rows, size_t ws_bytes);
 size_t dense_workspace_bytes(const DeviceLayer& L, int n, int h, int w, size_t most);
 // Activations in the dense kernel's own layout ("position rows", see kernels_dense.cu): the size of a
-// layer's input in it (0 = the shape has no such form), and the kernel that makes it from NCHW.
-size_t dense_rows_bytes(const DeviceLayer& L, int n, int h, int w, bool pool);
+// layer's input in it (0 = the shape has no such form; ws_bytes: the workspace its forward will have, under which
+// the plan is looked up), and the kernel that makes it from NCHW.
+size_t dense_rows_bytes(const DeviceLayer& L, int n, int h, int w, bool pool, size_t ws_bytes);
 cudaError_t launch_stage(const DeviceLayer& L, const void* x, void* rows, int n, int h, int w, bool pool,
                          cudaStream_t stream);
 struct DenseNext { int c_in, stride; bool pool; };   // the layer that reads the result as position rows

@@ -1,5 +1,7 @@
 """When launch plans of the dense kernel are worked out: planning is host work that a first pass pays for.
 The development build counts the plans made."""
+import threading
+
 import pytest
 import torch
 
@@ -35,8 +37,38 @@ def make(c_in, c_out, h, w, n=1, storage="f32", seed=1, stride=1):
 @pytest.mark.parametrize("storage", ["f32", "f16"])
 @pytest.mark.parametrize("flags", [B.KERNEL_TILED, B.KERNEL_SIMPLE, B.KERNEL_GENERIC_TAPS, B.ROWS4, B.ROWS8, B.CLUSTER])
 def test_a_pinned_kernel_needs_no_dense_plan(flags, storage):
-    layer, x = make(40, 24, 11, 19, storage=storage)
+    layer, x = make(40, 24, 11, 19 + flags.bit_length(), storage=storage)      # (a geometry that no other test has)
     y = torch.empty(layer.out_shape(x.shape), dtype=x.dtype, device="cuda")
     assert made(lambda: B.pconv_forward(layer.handle, x, layer.bias, y, flags | B.RELU)) == 0
     assert made(lambda: B.pconv_forward(layer.handle, x, layer.bias, y, B.RELU)) > 0       # (the choice needs some)
+    layer.close()
+
+
+def test_plans_are_shared_by_layers_of_the_same_geometry_and_by_threads():
+    first, x = make(48, 56, 13, 17)
+    other, _ = make(48, 56, 13, 17, seed=2)            # other weights, the same geometry
+    assert made(lambda: first.forward(x, split=True)) > 0
+    assert made(lambda: first.forward(x, split=True)) == 0
+    assert made(lambda: other.forward(x, split=True)) == 0
+    t = threading.Thread(target=lambda: made_there.append(made(lambda: other.forward(x, split=True))))
+    made_there = []
+    t.start()
+    t.join()
+    assert made_there == [0]
+    bigger, xb = make(48, 72, 13, 17)                  # another geometry
+    assert made(lambda: bigger.forward(xb, split=True)) > 0
+    torch.cuda.synchronize()
+    for l in (first, other, bigger):
+        l.close()
+
+
+def test_a_workspace_larger_than_needed_changes_no_plan():
+    layer, x = make(256, 64, 7, 9)
+    need = B.pconv_workspace_bytes(layer.handle, 1, 7, 9)
+    assert need > 0
+    y = torch.empty(layer.out_shape(x.shape), device="cuda")
+    for extra in (0, 256, 1 << 20):
+        ws = torch.zeros(need + extra, dtype=torch.uint8, device="cuda")
+        assert made(lambda: B.pconv_forward(layer.handle, x, layer.bias, y, B.RELU, workspace=ws)) == 0, extra
+        assert not ws.any()
     layer.close()
