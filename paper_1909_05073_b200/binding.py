@@ -98,6 +98,7 @@ def load(path):
         L.pconv_dev_withhold.argtypes = [ci, cu]
         L.pconv_dev_clear_status.argtypes = [vp]
         L.pconv_dev_dense_plans.restype = ctypes.c_longlong
+        L.pconv_dev_dense_plan.argtypes = [ci] * 10 + [ctypes.c_size_t, ci, ci, ip, ctypes.POINTER(ctypes.c_double)]
     L.pconv_status_str.argtypes = [ci]
     L.pconv_status_str.restype = ctypes.c_char_p
     L.pconv_stack_create.argtypes = [vp, vp, vp, ci, ci, ci, ci, cu, ctypes.POINTER(vp)]

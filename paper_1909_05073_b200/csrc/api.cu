@@ -341,6 +341,23 @@ extern "C" pconv_status pconv_dev_withhold(int chunk, unsigned spin_limit) {
 
 extern "C" long long pconv_dev_dense_plans(void) { return pconv::dense_plans_made(); }
 
+extern "C" pconv_status pconv_dev_dense_plan(int c_out, int c_in, int stride, int storage, int tap_mask, int n, int h_in,
+                                             int w_in, int pool, int rows, size_t ws_bytes, int cluster_sms, int prune,
+                                             int* fields, double* cycles) {
+  if (!fields || !cycles) return PCONV_ERR_NULL;
+  if (c_out <= 0 || c_in <= 0 || n <= 0 || h_in <= 0 || w_in <= 0 || (stride != 1 && stride != 2)) return PCONV_ERR_SHAPE;
+  pconv::DeviceLayer L;
+  std::memset(&L, 0, sizeof(L));
+  L.c_out = c_out;
+  L.c_in = c_in;
+  L.stride = stride;
+  L.storage = storage;
+  L.dense_rows = (c_out + 15) / 16 * 16;
+  L.tap_mask = tap_mask;
+  return pconv::dense_plan_of_shape(L, n, h_in, w_in, pool != 0, rows != 0, ws_bytes, cluster_sms, prune != 0, fields, cycles)
+             ? PCONV_OK : PCONV_ERR_UNSUPPORTED;
+}
+
 extern "C" pconv_status pconv_dev_clear_status(const pconv_handle* h) {
   if (!h) return PCONV_ERR_NULL;
   if (cudaDeviceSynchronize() != cudaSuccess || cudaMemset(h->d.err, 0, 4) != cudaSuccess ||

@@ -1551,18 +1551,20 @@ double mma_cycles(int n) { return n / 2.0 > 32.0 + n / 4.0 ? n / 2.0 : 32.0 + n 
 
 int round_up(int v, int m) { return (v + m - 1) / m * m; }
 
-// Geometry with `tiles` MMA tiles of nt filters per item, channel steps not cut; false if it does not fit.
-bool dense_geo(const DeviceLayer& L, int n, int h, int w, bool pool, bool p8, int tiles, int nt, DGeo* out) {
-  DGeo g = {};
+// Geometry in three steps, each kept while the next is tried with other values: of the map, with `tiles` MMA tiles
+// per item, and with nt filters per tile, channel steps not cut.  False where it does not fit.
+bool geo_of_map(const DeviceLayer& L, int n, int h, int w, bool pool, bool p8, DGeo* out) {
+  DGeo& g = *out;
+  g = DGeo{};
   const bool half = L.storage == PCONV_F16;
-  const int pieces = half ? 1 : 3, s = L.stride;
+  const int s = L.stride;
   g.n = n;
   g.h = h;
   g.w = w;
   g.c_in = L.c_in;
   g.c_out = L.c_out;
   const int ho = (h - 1) / s + 1, wo = (w - 1) / s + 1;     // of the convolution itself
-  if (pool && (s != 1 || tiles % 2)) return false;
+  if (pool && s != 1) return false;
   g.pool = pool ? 1 : 0;
   g.h_out = pool ? ho / 2 : ho;
   g.w_out = pool ? wo / 2 : wo;
@@ -1581,16 +1583,38 @@ bool dense_geo(const DeviceLayer& L, int n, int h, int w, bool pool, bool p8, in
   g.sy = (s == 2 || pool) ? 2 : 1;
   g.sx = s;
   g.planes = s == 2 ? 4 : (pool ? 2 : 1);
+  if ((long long)g.n_cells * g.cell_pos > 0x3FFFFFFF || (long long)n * L.c_in * h * w > 0x7FFFFFFF) return false;
+  // Producers' loads: as many pixels of a row as rows are aligned for (strips start off by one).
+  g.vec = 1;
+  if (g.strips == 1) g.vec = half && w % 4 == 0 ? 4 : (w % 2 == 0 ? 2 : 1);
+  g.row_planes = (s == 2 || pool) ? 2 : 1;
+  g.vec_cols = (s * g.pitch + g.vec - 1) / g.vec;
+  const Rows in = rows_of(L.c_in, s, n, h, w, pool);
+  if (p8 && in.plane_len < 0) return false;
+  if (p8) g.vec = 0;
+  g.in_plane_len = in.plane_len;
+  g.in_lead = in.lead;
+  g.rows = L.dense_rows;
+  g.n_taps = __builtin_popcount(L.tap_mask);
+  g.tps = half ? 3 : 1;
+  g.slots = (g.n_taps + g.tps - 1) / g.tps;
+  g.k_steps = (L.c_in + 15) / 16;
+  return true;
+}
+
+bool geo_of_tiles(const DeviceLayer& L, int tiles, DGeo* out) {
+  DGeo& g = *out;
+  const bool half = L.storage == PCONV_F16, pool = g.pool != 0;
+  if ((pool && tiles % 2) || (!half && tiles > 2)) return false;
   g.tiles = tiles;
   g.mpos = pool ? tiles * 64 : tiles * 128;
-  if ((long long)g.n_cells * g.cell_pos > 0x3FFFFFFF || (long long)n * L.c_in * h * w > 0x7FFFFFFF) return false;
   // taps: plane and shift
   int plane[kMaxT][9], shift[kMaxT][9], lo = 0, hi = 0, nk = 0;
   for (int t = 0; t < 9; ++t) {
     if (!(L.tap_mask >> t & 1)) continue;
     const int u = t / 3, v = t % 3;
     for (int j = 0; j < tiles; ++j) {
-      if (s == 2) {
+      if (L.stride == 2) {
         plane[j][nk] = (u == 1 ? 0 : 2) + (v == 1 ? 0 : 1);
         shift[j][nk] = (u == 0 ? -g.pitch : 0) + (v == 0 ? -1 : 0) + g.ox;
       } else if (pool) {
@@ -1606,44 +1630,35 @@ bool dense_geo(const DeviceLayer& L, int n, int h, int w, bool pool, bool p8, in
     }
     ++nk;
   }
-  g.n_taps = nk;
   g.lead = -lo;
   g.plane_pos = g.mpos + hi - lo;
   g.q_tot = g.planes * g.plane_pos;
   for (int j = 0; j < tiles; ++j)
     for (int t = 0; t < nk; ++t)
       g.tap_off[j][t] = plane[j][t] * g.plane_pos + g.lead + shift[j][t] + 128 * (pool ? j >> 1 : j);
-  // Producers' loads: as many pixels of a row as rows are aligned for (strips start off by one).
-  g.vec = 1;
-  if (g.strips == 1) g.vec = half && w % 4 == 0 ? 4 : (w % 2 == 0 ? 2 : 1);
-  g.row_planes = (s == 2 || pool) ? 2 : 1;
-  g.vec_cols = (s * g.pitch + g.vec - 1) / g.vec;
   g.vec_rows = (g.plane_pos + g.pitch - 2) / g.pitch + 1;
-  g.n_vec = p8 ? 0 : g.row_planes * g.vec_rows * g.vec_cols;
-  const Rows in = rows_of(L.c_in, s, n, h, w, pool);
-  if (p8 && in.plane_len < 0) return false;
-  if (p8) g.vec = 0;
-  g.in_plane_len = in.plane_len;
-  g.in_lead = in.lead;
-  g.rows = L.dense_rows;
+  g.n_vec = g.vec ? g.row_planes * g.vec_rows * g.vec_cols : 0;
+  g.a_bytes = (half ? 1 : 3) * 2 * g.q_tot * 16;
+  g.a_off = round_up(kHeader + kTables * g.n_vec * (int)sizeof(Load), 128);
+  return true;
+}
+
+bool geo_of_filters(const DeviceLayer& L, int nt, int sms, DGeo* out) {
+  DGeo& g = *out;
+  const bool half = L.storage == PCONV_F16, p8 = g.vec == 0;
+  const int tiles = g.tiles;
   g.nt = nt;
   g.n_ft = (g.rows + nt - 1) / nt;
   g.form3 = (!half && 3 * nt <= 256 && tiles * 3 * nt <= 512) ? 1 : 0;
   g.tile_cols = half ? nt : (g.form3 ? 3 : 2) * nt;
   g.n_buf = (half && tiles * nt <= 256) ? 2 : 1;
   if (tiles * g.tile_cols > 512 || nt > 128 || (!half && tiles * nt > (p8 ? 256 : 128))) return false;
-  if (!half && tiles > 2) return false;
   g.out_col = !half && tiles * (g.tile_cols + nt) <= 512 ? tiles * g.tile_cols : 0;
   g.out_stride = g.out_col ? nt : g.tile_cols;
   // the epilogue reads columns by 16, which may pass the end of a tile but not Tensor Memory's
   if (half && (g.n_buf == 2 ? 256 : 0) + (tiles - 1) * nt + nt / 2 + round_up(nt / 2, 16) > 512) return false;
   if (!half && (tiles - 1) * g.tile_cols + (g.form3 ? 2 : 1) * nt + nt / 2 + round_up(nt / 2, 16) > 512) return false;
-  g.tps = half ? 3 : 1;
-  g.slots = (nk + g.tps - 1) / g.tps;
-  g.k_steps = (L.c_in + 15) / 16;
-  g.a_bytes = pieces * 2 * g.q_tot * 16;
-  g.b_bytes = g.tps * pieces * 2 * nt * 16;
-  g.a_off = round_up(kHeader + kTables * g.n_vec * (int)sizeof(Load), 128);
+  g.b_bytes = g.tps * (half ? 1 : 3) * 2 * nt * 16;
   const int avail = kSmemLimit - g.a_off;
   // Activation stages first (two, so that one is filled while the other is read), then as many weight
   // slots as fit: what matters there is the time of the MMAs they cover against a copy's latency.
@@ -1658,8 +1673,7 @@ bool dense_geo(const DeviceLayer& L, int n, int h, int w, bool pool, bool p8, in
   const long long items = m_items * g.n_ft;
   if (items > 0x3FFFFF || items * g.k_steps > 0x3FFFFFFF) return false;
   g.n_tiles = (int)items;
-  g.grid = std::min(g.n_tiles, device_sm_count());
-  *out = g;
+  g.grid = std::min(g.n_tiles, sms);
   return true;
 }
 
@@ -1674,8 +1688,10 @@ size_t split_bytes(const DGeo& g) {
 // 36 bytes a cycle and SM from L2) or the staging of its activations, whichever is longest; an item ends with
 // its stores, which only the fp32 kernel and two accumulator sets overlap with the next item; a split adds
 // the exchange of partial sums.
-double dense_cycles(const DGeo& g, bool half) {
-  const double sms = device_sm_count();
+struct StepCost {
+  double step, epi;      // a channel step of an item, and its end
+};
+StepCost step_cost(const DGeo& g, bool half) {
   const int nt = g.nt;
   double tap = half ? mma_cycles(nt)
                     : (g.form3 ? mma_cycles(3 * nt) + mma_cycles(2 * nt) + mma_cycles(nt)
@@ -1688,11 +1704,16 @@ double dense_cycles(const DGeo& g, bool half) {
   if (wb > step) step = wb;
   if (conv > step) step = conv;
   step += 60;
-  const double epi = 600 + (half ? 8.0 : 16.0) * g.tiles * nt;
-  const double steps = g.split ? std::ceil((double)g.n_tiles * g.k_steps / g.grid)
-                               : std::ceil((double)g.n_tiles / g.grid) * g.k_steps;
-  const double segments = std::ceil(steps / g.k_steps);
-  double c = 4500 + steps * step + epi + (segments - 1) * (half && g.n_buf == 1 ? epi : 0.25 * epi);
+  return {step, 600 + (half ? 8.0 : 16.0) * g.tiles * nt};
+}
+long long ceil_div(long long a, long long b) { return (a + b - 1) / b; }
+double dense_cycles(const DGeo& g, const StepCost& cost, bool half, int sms) {
+  const int nt = g.nt;
+  const double epi = cost.epi;
+  const long long steps = g.split ? ceil_div((long long)g.n_tiles * g.k_steps, g.grid)
+                                  : ceil_div(g.n_tiles, g.grid) * g.k_steps;
+  const long long segments = ceil_div(steps, g.k_steps);
+  double c = 4500 + steps * cost.step + epi + (segments - 1) * (half && g.n_buf == 1 ? epi : 0.25 * epi);
   if (g.split) {
     // A part hands its sums over, inside a cluster or added to the workspace.  Measured on layers of 49 to
     // 3136 positions: a cluster's exchange 5000-6000 cycles, more where large clusters have to wait for
@@ -1704,17 +1725,23 @@ double dense_cycles(const DGeo& g, bool half) {
   }
   return c;
 }
+// What no way of cutting these tiles can fall below: all steps spread evenly over all SMs.
+double least_cycles(const DGeo& g, const StepCost& cost, int sms) {
+  return 4500 + ceil_div((long long)g.n_tiles * g.k_steps, sms) * cost.step + cost.epi;
+}
 
-int max_clusters(bool half, int parts);   // below: needs the kernels
+int max_clusters(int dev, bool half, int parts);   // below: needs the kernels
 #ifdef PCONV_DEV
 std::atomic<long long> g_plans_made{0};
 #endif
 
-// The geometry of a launch: the cheapest by the estimate.  ws_bytes: workspace the caller has.
-bool dense_plan(const DeviceLayer& L, int n, int h, int w, bool pool, bool p8, size_t ws_bytes, DGeo* out, double* cycles) {
-  if (!L.wdense || n <= 0 || h <= 0 || w <= 0) return false;
+// The geometry of a launch: the cheapest by the estimate.  ws_bytes: workspace the caller has; sms, clusters(parts):
+// the device's.  `prune`: what cannot become the cheapest is left out before its ways of cutting are gone through,
+// which changes no plan.
+template <typename Clusters>
+bool dense_plan(const DeviceLayer& L, int n, int h, int w, bool pool, bool p8, size_t ws_bytes, int sms, Clusters clusters,
+                bool prune, DGeo* out, double* cycles) {
   const bool half = L.storage == PCONV_F16;
-  const int sms = device_sm_count();
   bool found = false;
   double best = 0.0;
 #ifdef PCONV_DEV
@@ -1722,53 +1749,62 @@ bool dense_plan(const DeviceLayer& L, int n, int h, int w, bool pool, bool p8, s
   int force[4] = {0, 0, 0, 0};
   if (const char* e = getenv("PCONV_FORCE_DENSE")) sscanf(e, "%d,%d,%d,%d", &force[0], &force[1], &force[2], &force[3]);
 #endif
+  DGeo of_tiles[3];                              // 1, 2 and 4 tiles
+  bool fits[3];
+  if (!geo_of_map(L, n, h, w, pool, p8, &of_tiles[0])) return false;
+  of_tiles[1] = of_tiles[2] = of_tiles[0];
+  for (int t = 0; t < 3; ++t) fits[t] = geo_of_tiles(L, 1 << t, &of_tiles[t]);
   int last_nt = 0;
-  for (int parts = (L.dense_rows + 127) / 128; parts <= L.dense_rows / 16; parts = parts < 4 ? parts + 1 : parts * 2) {
-    const int nt = round_up((L.dense_rows + parts - 1) / parts, 16);
+  for (int cut = (L.dense_rows + 127) / 128; cut <= L.dense_rows / 16; cut = cut < 4 ? cut + 1 : cut * 2) {
+    const int nt = round_up((L.dense_rows + cut - 1) / cut, 16);
     if (nt == last_nt || nt > 128) continue;
     last_nt = nt;
     if (nt < 32 && L.dense_rows > 16) break;
-    for (int tiles = 1; tiles <= kMaxT; tiles *= 2) {
-      DGeo g;
-      if (!dense_geo(L, n, h, w, pool, p8, tiles, nt, &g)) continue;
+    for (int t = 0; t < 3; ++t) {
+      DGeo g = of_tiles[t];
+      if (!fits[t] || !geo_of_filters(L, nt, sms, &g)) continue;
+      const StepCost cost = step_cost(g, half);
+      if (prune && found && least_cycles(g, cost, sms) >= best) continue;
       // Whole tiles only (v = 0); or the line of steps cut evenly among all SMs (1); or each tile cut in
       // v / 2 parts, a CTA's each: in the workspace (even v; equal parts, which end together) or, up to
       // eight, by a cluster, which needs none.
+      const int whole = g.grid;
       for (int v = 0; v <= 2 * (g.k_steps / kMinSteps) + 1; ++v) {
-        DGeo c = g;
         const int parts = v < 2 ? v : v / 2;
+        g.grid = whole;
+        g.split = g.cluster = 0;
         if (parts == 1) {
           if (v != 1 || g.n_tiles % sms == 0 || g.k_steps < 2 * kMinSteps) continue;
-          c.grid = (int)std::min<long long>(sms, (long long)g.n_tiles * (g.k_steps / kMinSteps));
-          c.split = 1;
+          g.grid = (int)std::min<long long>(sms, (long long)g.n_tiles * (g.k_steps / kMinSteps));
+          g.split = 1;
         } else if (parts > 1) {
           if ((long long)g.n_tiles * parts > sms || g.k_steps < kMinSteps * parts) break;
-          c.grid = g.n_tiles * parts;
-          c.split = 1;
-          c.cluster = v & 1;
-          if (!c.cluster && g.k_steps % parts != 0) continue;
-          if (c.cluster && (parts > 8 || g.n_tiles > max_clusters(half, parts) ||
-                            tiles * nt * 512 > g.a_stages * g.a_bytes + g.b_slots * g.b_bytes))
+          g.grid = g.n_tiles * parts;
+          g.split = 1;
+          g.cluster = v & 1;
+          if (!g.cluster && g.k_steps % parts != 0) continue;
+          if (g.cluster && (parts > 8 || g.n_tiles > clusters(parts) ||
+                            g.tiles * nt * 512 > g.a_stages * g.a_bytes + g.b_slots * g.b_bytes))
             continue;
         }
-        if (split_bytes(c) > ws_bytes) continue;
-        const int all = c.split ? c.n_tiles * c.k_steps : c.n_tiles;
-        c.share = all / c.grid;
-        c.share_more = all % c.grid;
-        c.parts = c.cluster ? parts : c.split && c.share_more == 0 && c.k_steps % c.share == 0 ? c.k_steps / c.share : 0;
-        double cost = dense_cycles(c, half);
+        if (split_bytes(g) > ws_bytes) continue;
+        const int all = g.split ? g.n_tiles * g.k_steps : g.n_tiles;
+        g.share = all / g.grid;
+        g.share_more = all % g.grid;
+        g.parts = g.cluster ? parts : g.split && g.share_more == 0 && g.k_steps % g.share == 0 ? g.k_steps / g.share : 0;
+        double c = dense_cycles(g, cost, half, sms);
 #ifdef PCONV_DEV
-        if (force[0] && (force[0] != tiles || force[1] != nt || force[2] != c.grid || force[3] != c.cluster)) cost += 1e12;
+        if (force[0] && (force[0] != g.tiles || force[1] != nt || force[2] != g.grid || force[3] != g.cluster)) c += 1e12;
 #endif
-        if (!found || cost < best) {
+        if (!found || c < best) {
           found = true;
-          best = cost;
-          *out = c;
+          best = c;
+          *out = g;
         }
       }
     }
   }
-  if (found && cycles) *cycles = best;
+  if (found) *cycles = best;
   return found;
 }
 
@@ -1826,7 +1862,9 @@ Plan find_plan(const DeviceLayer& L, int n, int h, int w, bool pool, bool p8, si
   DGeo& g = made.geo;
   made.key = k;
   made.most = ws_bytes;
-  made.plan.found = dense_plan(L, n, h, w, pool, p8, ws_bytes, &g, &made.plan.cycles);
+  const bool half = L.storage == PCONV_F16;
+  made.plan.found = dense_plan(L, n, h, w, pool, p8, ws_bytes, device_sm_count(),
+                               [&](int parts) { return max_clusters(dev, half, parts); }, true, &g, &made.plan.cycles);
   if (made.plan.found) made.plan.need = split_bytes(g);
   made.plan.n_tiles = g.n_tiles;
   made.plan.n_ft = g.n_ft;
@@ -1879,14 +1917,10 @@ __global__ void __launch_bounds__(128) dense_weights_kernel(const DeviceLayer L)
 }
 
 // Clusters of `parts` CTAs that the device holds at once (one CTA per SM, the SMs of a cluster inside one
-// GPC); asked once per size and device.  Without a device: none.
-int max_clusters(bool half, int parts) {
+// GPC); asked once per size and device (`dev`: the current one).  Without a device: none.
+int max_clusters(int dev, bool half, int parts) {
   static std::atomic<int> known[64][2][9];
-  int dev = -1;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
-    cudaGetLastError();
-    return 0;
-  }
+  if (dev < 0 || dev >= 64) return 0;
   std::atomic<int>& slot = known[dev][half ? 1 : 0][parts];
   int v = slot.load();
   if (v) return v - 1;
@@ -2065,6 +2099,16 @@ DensePath dense_path(const DeviceLayer& L, int n, int h, int w, bool pool, RowsF
 }
 
 #ifdef PCONV_DEV
+bool dense_plan_of_shape(const DeviceLayer& L, int n, int h, int w, bool pool, bool p8, size_t ws_bytes, int cluster_sms,
+                         bool prune, int* out, double* cycles) {
+  DGeo g = {};
+  if (!dense_plan(L, n, h, w, pool, p8, ws_bytes, 148, [&](int parts) { return cluster_sms / parts; }, prune, &g, cycles))
+    return false;
+  const int f[14] = {g.tiles, g.nt, g.grid, g.split, g.cluster, g.parts, g.n_tiles, g.k_steps, g.a_stages, g.b_slots,
+                     g.b_off + g.b_slots * g.b_bytes, g.tiles * g.tile_cols, (int)split_bytes(g), g.share};
+  for (int i = 0; i < 14; ++i) out[i] = f[i];
+  return true;
+}
 long long dense_plans_made() { return g_plans_made.load(); }
 
 cudaError_t dense_set_withhold(int step, unsigned spin_limit) {

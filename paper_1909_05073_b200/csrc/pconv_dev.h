@@ -36,6 +36,15 @@ pconv_status pconv_dev_withhold(int chunk, unsigned spin_limit);
  * plan already made adds none). */
 long long pconv_dev_dense_plans(void);
 
+/* The dense kernel's plan for a shape on a device of 148 SMs of which `cluster_sms` can hold clusters (host
+ * arithmetic, needs no device).  rows: the input is position rows.  prune = 0: every candidate is costed.
+ * fields[14]: tiles of an item, filters of a tile, CTAs, split, cluster, equal parts of a tile, tiles, channel steps,
+ * activation stages, weight slots, shared memory bytes, Tensor Memory columns of an accumulator set, workspace
+ * bytes, a CTA's share.  PCONV_ERR_UNSUPPORTED if there is none. */
+pconv_status pconv_dev_dense_plan(int c_out, int c_in, int stride, int storage, int tap_mask, int n, int h_in, int w_in,
+                                  int pool, int rows, size_t ws_bytes, int cluster_sms, int prune, int* fields,
+                                  double* cycles);
+
 /* Clears the handle's sticky status word (pconv_device_status reports PCONV_OK again until the
  * next abandoned wait).  Synchronises the device. */
 pconv_status pconv_dev_clear_status(const pconv_handle* h);

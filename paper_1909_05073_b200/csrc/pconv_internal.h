@@ -165,6 +165,8 @@ bool tiled_plan(const DeviceLayer& L, int n, int h, int w, bool generic_taps, bo
 cudaError_t dev_set_withhold(int chunk, unsigned spin_limit);     // see pconv_dev.h
 cudaError_t dense_set_withhold(int step, unsigned spin_limit);
 long long dense_plans_made();
+bool dense_plan_of_shape(const DeviceLayer& L, int n, int h, int w, bool pool, bool p8, size_t ws_bytes, int cluster_sms,
+                         bool prune, int* out, double* cycles);
 #endif
 // chains: several consecutive layers of a stack in one persistent launch (kernels_tiled.cu)
 bool chain_layer_ok(const DeviceLayer& L, int n, int h, int w, bool pool, long long* ctas);
