@@ -153,8 +153,9 @@ extern "C" pconv_status pconv_scratch_bytes(const pconv_handle* h, int n, int h_
   if (!h || !bytes) return PCONV_ERR_NULL;
   if (n < 0 || h_in <= 0 || w_in <= 0) return PCONV_ERR_SHAPE;
   *bytes = 0;
-  for (int pool = 0; n > 0 && pool < 2; ++pool)
-    *bytes = std::max(*bytes, dense_rows_bytes(h->d, n, h_in, w_in, pool != 0, pconv::kMaxSplitBytes));
+  // whichever form a forward of this shape may take: with the workspace it may have, or without one
+  for (int v = 0; n > 0 && v < 4; ++v)
+    *bytes = std::max(*bytes, dense_scratch_bytes(h->d, n, h_in, w_in, (v & 1) != 0, (v & 2) ? 0 : pconv::kMaxSplitBytes));
   return PCONV_OK;
 }
 
@@ -209,9 +210,8 @@ static pconv_status forward_impl(const pconv_handle* h, const void* x, const flo
   const size_t dense_ws_bytes = dense_ws ? ws_bytes : 0;
   bool dense = false, staged = false;
   if (sel == 0 && rmode == 0 && !cluster) {
-    const size_t rows = scratch ? dense_rows_bytes(L, n, h_in, w_in, pool, dense_ws_bytes) : 0;
-    const DensePath path = dense_path(L, n, h_in, w_in, pool, rows > 0 && rows <= scratch_bytes ? kRowsStaged : kNoRows,
-                                      dense_ws_bytes);
+    const bool room = scratch && dense_rows_bytes(L, n, h_in, w_in, pool) <= scratch_bytes;
+    const DensePath path = dense_path(L, n, h_in, w_in, pool, room ? kRowsStaged : kNoRows, dense_ws_bytes);
     staged = path == kFromRows;
     dense = path != kNotDense || (!pool && batch_on_tensor_cores(L, n, h_in, w_in, dense_ws_bytes));
   }
@@ -542,16 +542,14 @@ static bool build_rows(pconv_stack* s) {
     for (const pconv_stack::Chain& c : *s->chains) chained = chained || (i >= c.begin && i < c.end);
     const bool pool = s->pool[i] != 0;
     if (!chained) {
-      const size_t bytes = pconv::dense_rows_bytes(L, s->n, ch, cw, pool, ws_bytes);
-      const bool given = bytes > 0 && i > 0 && (*s->path)[i - 1] != pconv::kNotDense;
-      (*s->path)[i] = pconv::dense_path(L, s->n, ch, cw, pool,
-                                        given ? pconv::kRowsGiven : bytes > 0 ? pconv::kRowsStaged : pconv::kNoRows, ws_bytes);
+      const bool given = i > 0 && (*s->path)[i - 1] != pconv::kNotDense && pconv::dense_takes_rows(L, s->n, ch, cw, pool, ws_bytes);
+      (*s->path)[i] = pconv::dense_path(L, s->n, ch, cw, pool, given ? pconv::kRowsGiven : pconv::kRowsStaged, ws_bytes);
       if ((*s->path)[i] == pconv::kNotDense && batch_on_tensor_cores(L, s->n, ch, cw, ws_bytes) &&
           pconv::dense_supported(L, s->n, ch, cw, pool, ws_bytes))
         (*s->path)[i] = pconv::kFromNchw;
       if ((*s->path)[i] == pconv::kFromRows) {
         at[i] = total + 1;
-        total += (bytes + 255) & ~(size_t)255;
+        total += (pconv::dense_rows_bytes(L, s->n, ch, cw, pool) + 255) & ~(size_t)255;
       }
     }
     ch = (ch - 1) / L.stride + 1;

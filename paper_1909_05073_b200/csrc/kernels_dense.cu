@@ -2005,9 +2005,16 @@ size_t dense_workspace_bytes(const DeviceLayer& L, int n, int h, int w, size_t m
   return need;
 }
 
-size_t dense_rows_bytes(const DeviceLayer& L, int n, int h, int w, bool pool, size_t ws_bytes) {
-  if (!find_plan(L, n, h, w, pool, true, ws_bytes).found) return 0;
+bool dense_takes_rows(const DeviceLayer& L, int n, int h, int w, bool pool, size_t ws_bytes) {
+  return find_plan(L, n, h, w, pool, true, ws_bytes).found;
+}
+
+size_t dense_rows_bytes(const DeviceLayer& L, int n, int h, int w, bool pool) {
   return rows_bytes(rows_of(L.c_in, L.stride, n, h, w, pool), L.storage == PCONV_F16);
+}
+
+size_t dense_scratch_bytes(const DeviceLayer& L, int n, int h, int w, bool pool, size_t ws_bytes) {
+  return dense_path(L, n, h, w, pool, kRowsStaged, ws_bytes) == kFromRows ? dense_rows_bytes(L, n, h, w, pool) : 0;
 }
 
 cudaError_t launch_stage(const DeviceLayer& L, const void* x, void* rows, int n, int h, int w, bool pool,

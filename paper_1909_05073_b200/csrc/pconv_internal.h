@@ -141,10 +141,12 @@ enum RowsFrom { kNoRows, kRowsStaged, kRowsGiven };    // position rows: no room
 enum DensePath { kNotDense, kFromNchw, kFromRows };
 DensePath dense_path(const DeviceLayer& L, int n, int h, int w, bool pool, RowsFrom rows, size_t ws_bytes);
 size_t dense_workspace_bytes(const DeviceLayer& L, int n, int h, int w, size_t most);
-// Activations in the dense kernel's own layout ("position rows", see kernels_dense.cu): the size of a
-// layer's input in it (0 = the shape has no such form; ws_bytes: the workspace its forward will have, under which
-// the plan is looked up), and the kernel that makes it from NCHW.
-size_t dense_rows_bytes(const DeviceLayer& L, int n, int h, int w, bool pool, size_t ws_bytes);
+// Activations in the dense kernel's own layout ("position rows", see kernels_dense.cu): whether the kernel
+// takes a layer's input in it, the input's size, the size of it that a forward from NCHW with this workspace would use
+// (0 = it would not), and the kernel that makes it from NCHW.
+bool dense_takes_rows(const DeviceLayer& L, int n, int h, int w, bool pool, size_t ws_bytes);
+size_t dense_rows_bytes(const DeviceLayer& L, int n, int h, int w, bool pool);
+size_t dense_scratch_bytes(const DeviceLayer& L, int n, int h, int w, bool pool, size_t ws_bytes);
 cudaError_t launch_stage(const DeviceLayer& L, const void* x, void* rows, int n, int h, int w, bool pool,
                          cudaStream_t stream);
 struct DenseNext { int c_in, stride; bool pool; };   // the layer that reads the result as position rows

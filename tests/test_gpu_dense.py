@@ -1,7 +1,8 @@
 """GPU parity of the dense tensor-core kernel for both storage types, where it can go wrong: tiles of 128
 positions and up to 128 filters that are just missed or just passed, channel counts around a step of
 16, maps of one pixel and of one row, column strips, both strides, the fused pool, tap sets smaller than
-nine, tiles shared by several thread blocks, and both forms of the input (NCHW and position rows)."""
+nine, tiles shared by several thread blocks, and both forms of the input (NCHW and position rows).  The
+development build pins the kernel and the form; the layers' own choice is tried beside them."""
 import numpy as np
 import pytest
 import torch
@@ -16,9 +17,11 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.fixture(scope="module", autouse=True)
-def _built():
-    pbuild.build()
-    B.lib()
+def dev_library():
+    old = B.use_library(pbuild.build(dev=True))
+    yield
+    B.use_library(None)
+    B._lib = old
 
 
 CASES = [  # (c_in, c_out, h, w, n, stride, patterns)
@@ -41,9 +44,10 @@ CASES = [  # (c_in, c_out, h, w, n, stride, patterns)
 
 @pytest.mark.parametrize("storage", ["f32", "f16"])
 @pytest.mark.parametrize("case", CASES, ids=lambda c: "x".join(str(v) for v in c[:6]))
-def test_dense_kernel_matches_the_oracle_from_both_forms_of_the_input(case, storage):
+def test_dense_kernel_matches_the_oracle_from_both_forms_of_the_input(case, storage, monkeypatch):
     c_in, c_out, h, w, n, stride, pats = case
-    spec = synth.LayerSpec("t", c_in, c_out, h, w, stride, 0.7, (1.0 / len(pats),) * len(pats))
+    # (a layer without any kernel has no dense weights: the smallest one keeps its only kernel)
+    spec = synth.LayerSpec("t", c_in, c_out, h, w, stride, 1.0 if c_in * c_out == 1 else 0.7, (1.0 / len(pats),) * len(pats))
     wt, bias, _ = synth.gen_weights(spec, 300 + c_in + c_out, pats)
     x = synth.gen_input(spec, n, 300 + c_in)
     layer = B.Layer(wt, pats, stride, B.F16 if storage == "f16" else B.F32, bias)
@@ -55,13 +59,23 @@ def test_dense_kernel_matches_the_oracle_from_both_forms_of_the_input(case, stor
         want = oracle.maxpool2x2(ref) if pool else ref
         for split in (False, True):
             ws = layer.workspace(xt.shape) if split else None
-            for scratch in (None, layer.scratch(xt.shape)):
-                y = Guarded(want.shape, xt.dtype, fill=float("nan"))
-                B.pconv_forward(layer.handle, xt, layer.bias, y.t, B.RELU | (B.POOL2X2 if pool else 0), workspace=ws,
-                                scratch=scratch)
-                y.check("output")
-                check_close(y.t.float().cpu().numpy(), want, storage,
-                            "pool=%s split=%s rows=%s" % (pool, split, scratch is not None))
+            for form in ("chosen", "nchw", "rows"):
+                with monkeypatch.context() as m:
+                    if form != "chosen":
+                        m.setenv("PCONV_FORCE_DENSE", "0,0,0,0")
+                        m.setenv("PCONV_FORCE_ROWS", "1" if form == "rows" else "0")
+                    need = B.pconv_scratch_bytes(layer.handle, n, h, w)
+                    assert need > 0 if form == "rows" else need == 0 or form == "chosen"
+                    scratch = Guarded((need,), torch.uint8, fill=0xFF) if need else None     # (NaNs, where nothing is staged)
+                    y = Guarded(want.shape, xt.dtype, fill=float("nan"))
+                    B.pconv_forward(layer.handle, xt, layer.bias, y.t, B.RELU | (B.POOL2X2 if pool else 0), workspace=ws,
+                                    scratch=scratch and scratch.t)
+                    y.check("output")
+                    if scratch:
+                        scratch.check("scratch")
+                        # (stride 2 with a pool has no dense form: the tiled kernel runs)
+                        assert form != "rows" or (pool and stride == 2) or (scratch.t != 0xFF).any()
+                check_close(y.t.float().cpu().numpy(), want, storage, "pool=%s split=%s %s" % (pool, split, form))
         if layer._ws is not None:
             assert not layer._ws.any()
     assert B.pconv_device_status(layer.handle) == (0, 0)
@@ -70,9 +84,11 @@ def test_dense_kernel_matches_the_oracle_from_both_forms_of_the_input(case, stor
 
 @pytest.mark.parametrize("storage", ["f32", "f16"])
 @pytest.mark.parametrize("n,h,w", [(1, 32, 32), (3, 37, 29), (40, 8, 8)])
-def test_stack_that_hands_position_rows_from_layer_to_layer(n, h, w, storage):
+def test_stack_that_hands_position_rows_from_layer_to_layer(n, h, w, storage, monkeypatch):
     """Layers of ragged widths, pools and a stride-2 layer: every kind of row layout is written by one
-    layer and read by the next."""
+    layer and read by the next (the dense kernel on rows pinned: six launches, one of which stages)."""
+    monkeypatch.setenv("PCONV_FORCE_DENSE", "0,0,0,0")
+    monkeypatch.setenv("PCONV_FORCE_ROWS", "1")
     chans, pools, strides = [17, 40, 100, 256, 260, 20], [0, 1, 0, 0, 1], [1, 1, 2, 1, 1]
     dt = torch.float16 if storage == "f16" else torch.float32
     specs = [synth.LayerSpec("l%d" % i, chans[i], chans[i + 1], h, w, strides[i], 0.4, sigma=None) for i in range(5)]
@@ -86,6 +102,7 @@ def test_stack_that_hands_position_rows_from_layer_to_layer(n, h, w, storage):
             a = a.astype(np.float16).astype(np.float32)
         a = oracle.maxpool2x2(a) if pools[i] else a
     stack = B.Stack(layers, pools, n, h, w, B.RELU)
+    assert stack.launches() == 6
     y = Guarded(stack.out_shape, dt, fill=float("nan"))
     for _ in range(2):
         stack.forward(torch.from_numpy(x).cuda().to(dt), y.t)

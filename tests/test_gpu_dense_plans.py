@@ -72,3 +72,29 @@ def test_a_workspace_larger_than_needed_changes_no_plan():
         assert made(lambda: B.pconv_forward(layer.handle, x, layer.bias, y, B.RELU, workspace=ws)) == 0, extra
         assert not ws.any()
     layer.close()
+
+
+@pytest.mark.parametrize("case", [
+    (512, 512, 14, 14, 64, 1, "f32"), (512, 512, 28, 28, 16, 2, "f32"), (64, 64, 56, 56, 1, 1, "f32"),
+    (256, 256, 28, 28, 8, 1, "f32"), (130, 75, 57, 61, 9, 2, "f16"), (256, 256, 56, 56, 1, 1, "f32"),
+    (64, 64, 32, 32, 64, 1, "f16"), (512, 512, 4, 4, 64, 1, "f16"), (33, 60, 19, 23, 3, 1, "f16"),
+], ids=lambda c: "x".join(str(v) for v in c))
+def test_scratch_is_asked_for_where_a_forward_uses_it_and_nowhere_else(case):
+    c_in, c_out, h, w, n, stride, storage = case
+    layer, x = make(c_in, c_out, h, w, n, storage, 3, stride)
+    x.uniform_(0.5, 1.5)
+    need = B.pconv_scratch_bytes(layer.handle, n, h, w)
+    ws = layer.workspace(x.shape)
+    touched = 0
+    for pool in (False, True) if stride == 1 else (False,):
+        for workspace in {id(ws): ws, id(None): None}.values():
+            room = torch.full((256 << 20,), 0xA5, dtype=torch.uint8, device="cuda")
+            _, co, ho, wo = layer.out_shape(x.shape)
+            y = torch.empty((n, co, ho // 2, wo // 2) if pool else (n, co, ho, wo), dtype=x.dtype, device="cuda")
+            B.pconv_forward(layer.handle, x, layer.bias, y, B.RELU | (B.POOL2X2 if pool else 0), workspace=workspace, scratch=room)
+            used = (room != 0xA5).nonzero()
+            touched = max(touched, int(used.max()) + 1 if len(used) else 0)
+    assert touched <= need, "a forward used more than was asked for"
+    assert (touched > 0) == (need > 0), "%d bytes asked for, %d used" % (need, touched)
+    assert B.pconv_device_status(layer.handle) == (0, 0)
+    layer.close()
