@@ -49,6 +49,10 @@ extern "C" const char* pconv_status_str(pconv_status s) {
   return "unknown status";
 }
 
+// With one of these the library does not choose between the kernels.
+static constexpr unsigned kPinsKernel = PCONV_KERNEL_SIMPLE | PCONV_KERNEL_TILED | PCONV_KERNEL_GENERIC_TAPS |
+                                        PCONV_KERNEL_TENSOR | PCONV_ROWS4 | PCONV_ROWS8 | PCONV_CLUSTER | PCONV_STAGE_BULK;
+
 // What a caller pinned for the tiled kernel: rows per lane (0 = the planner chooses) and the
 // bulk-copy staging.
 static int rows_mode(unsigned flags) {
@@ -71,7 +75,8 @@ static bool batch_on_tensor_cores(const pconv::DeviceLayer& L, int n, int h, int
 // the caller pins for the tiled kernel (0 = the planner's choice), -1 = whatever it may pin.  The dense
 // kernel makes do with what it gets: `most_dense` bounds what it asks for.
 static size_t workspace_need(const pconv::DeviceLayer& L, int n, int h_in, int w_in, int rmode, size_t most_dense) {
-  size_t need = dense_workspace_bytes(L, n, h_in, w_in, most_dense);
+  size_t need = std::max(dense_workspace_bytes(L, n, h_in, w_in, false, kRowsStaged, most_dense),
+                         dense_workspace_bytes(L, n, h_in, w_in, true, kRowsStaged, most_dense));
   for (int r = 0; r <= 8; r += 4)
     for (int bulk = 0; bulk <= pconv::kPinBulk; bulk += pconv::kPinBulk) {
       if (rmode >= 0 && (r | bulk) != rmode) continue;
@@ -209,7 +214,7 @@ static pconv_status forward_impl(const pconv_handle* h, const void* x, const flo
   void* dense_ws = repro ? nullptr : ws;
   const size_t dense_ws_bytes = dense_ws ? ws_bytes : 0;
   bool dense = false, staged = false;
-  if (sel == 0 && rmode == 0 && !cluster) {
+  if (!(flags & kPinsKernel)) {
     const bool room = scratch && dense_rows_bytes(L, n, h_in, w_in, pool) <= scratch_bytes;
     const DensePath path = dense_path(L, n, h_in, w_in, pool, room ? kRowsStaged : kNoRows, dense_ws_bytes);
     staged = path == kFromRows;
@@ -529,9 +534,7 @@ static bool build_rows(pconv_stack* s) {
   s->rows = new (std::nothrow) std::vector<void*>(s->n_layers, nullptr);
   s->path = new (std::nothrow) std::vector<pconv::DensePath>(s->n_layers, pconv::kNotDense);
   if (!s->rows || !s->path) return false;
-  const unsigned pinned = PCONV_KERNEL_SIMPLE | PCONV_KERNEL_TILED | PCONV_KERNEL_GENERIC_TAPS | PCONV_KERNEL_TENSOR |
-                          PCONV_ROWS4 | PCONV_ROWS8 | PCONV_CLUSTER | PCONV_STAGE_BULK;
-  if (s->flags & pinned) return true;
+  if (s->flags & kPinsKernel) return true;
   const size_t ws_bytes = (s->flags & PCONV_REPRODUCIBLE) ? 0 : s->ws_bytes;
   std::vector<size_t> at(s->n_layers, 0);
   size_t total = 0;
@@ -603,9 +606,13 @@ extern "C" pconv_status pconv_stack_create(const pconv_handle* const* layers,
       pconv_stack_free(s);
       return PCONV_ERR_SHAPE;
     }
-    const size_t wsb = tiled_workspace_bytes(L, n, ch, cw, rows_mode(flags)), wsd = dense_workspace_bytes(L, n, ch, cw, pconv::kMaxSplitBytes);
-    if (wsb > s->ws_bytes) s->ws_bytes = wsb;
-    if (wsd > s->ws_bytes) s->ws_bytes = wsd;
+    s->ws_bytes = std::max(s->ws_bytes, tiled_workspace_bytes(L, n, ch, cw, rows_mode(flags)));
+    if (flags & PCONV_KERNEL_TENSOR)      // (reads NCHW, and its pool is a kernel of its own)
+      s->ws_bytes = std::max(s->ws_bytes, dense_workspace_bytes(L, n, ch, cw, false, pconv::kNoRows, pconv::kMaxSplitBytes));
+    else if (!(flags & kPinsKernel))
+      s->ws_bytes = std::max(s->ws_bytes, dense_workspace_bytes(L, n, ch, cw, s->pool[i] != 0,
+                                                                i > 0 ? pconv::kRowsGiven : pconv::kRowsStaged,
+                                                                pconv::kMaxSplitBytes));
     ch = (ch - 1) / L.stride + 1;
     cw = (cw - 1) / L.stride + 1;
     cc = L.c_out;

@@ -1997,11 +1997,10 @@ bool dense_supported(const DeviceLayer& L, int n, int h, int w, bool pool, size_
   return find_plan(L, n, h, w, pool, false, ws_bytes).found;
 }
 
-size_t dense_workspace_bytes(const DeviceLayer& L, int n, int h, int w, size_t most) {
-  size_t need = 0;
-  for (int v = 0; v < 4; ++v) {
-    need = std::max(need, find_plan(L, n, h, w, v & 1, v & 2, most).need);
-  }
+size_t dense_workspace_bytes(const DeviceLayer& L, int n, int h, int w, bool pool, RowsFrom rows, size_t most) {
+  size_t need = find_plan(L, n, h, w, pool, false, most).need;
+  if (rows == kRowsGiven || dense_path(L, n, h, w, pool, rows, most) == kFromRows)
+    need = std::max(need, find_plan(L, n, h, w, pool, true, most).need);
   return need;
 }
 
@@ -2094,13 +2093,13 @@ DensePath dense_path(const DeviceLayer& L, int n, int h, int w, bool pool, RowsF
       path = kFromNchw;
     }
   }
-  if (rows != kNoRows) {
+  const double staging = rows != kRowsStaged ? 0.0 :
+      5500.0 + ((double)rows_bytes(rows_of(L.c_in, L.stride, n, h, w, pool), half) +
+                (double)n * L.c_in * h * w * (half ? 2 : 4)) / 2200.0;
+  // (no plan where staging the input alone leaves too little: no launch is estimated below 5100 cycles)
+  if (rows != kNoRows && staging + 5100.0 < best) {
     const Plan e = find_plan(L, n, h, w, pool, true, ws_bytes);
-    double cycles = cycles_of(e);
-    if (e.found && rows == kRowsStaged)
-      cycles += 5500.0 + ((double)rows_bytes(rows_of(L.c_in, L.stride, n, h, w, pool), half) +
-                          (double)n * L.c_in * h * w * (half ? 2 : 4)) / 2200.0;
-    if (e.found && cycles < best) path = kFromRows;
+    if (e.found && cycles_of(e) + staging < best) path = kFromRows;
   }
   return path;
 }

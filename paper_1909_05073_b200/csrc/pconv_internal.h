@@ -140,7 +140,8 @@ bool dense_supported(const DeviceLayer& L, int n, int h, int w, bool pool, size_
 enum RowsFrom { kNoRows, kRowsStaged, kRowsGiven };    // position rows: no room, to be staged, already there
 enum DensePath { kNotDense, kFromNchw, kFromRows };
 DensePath dense_path(const DeviceLayer& L, int n, int h, int w, bool pool, RowsFrom rows, size_t ws_bytes);
-size_t dense_workspace_bytes(const DeviceLayer& L, int n, int h, int w, size_t most);
+// Workspace of the forms that a forward may take with up to `most` bytes of it.
+size_t dense_workspace_bytes(const DeviceLayer& L, int n, int h, int w, bool pool, RowsFrom rows, size_t most);
 // Activations in the dense kernel's own layout ("position rows", see kernels_dense.cu): whether the kernel
 // takes a layer's input in it, the input's size, the size of it that a forward from NCHW with this workspace would use
 // (0 = it would not), and the kernel that makes it from NCHW.

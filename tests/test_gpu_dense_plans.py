@@ -98,3 +98,26 @@ def test_scratch_is_asked_for_where_a_forward_uses_it_and_nowhere_else(case):
     assert (touched > 0) == (need > 0), "%d bytes asked for, %d used" % (need, touched)
     assert B.pconv_device_status(layer.handle) == (0, 0)
     layer.close()
+
+
+def test_a_first_forward_plans_only_what_it_may_run():
+    """The sizes of workspace and scratch, which are asked for before it, need NCHW plans (plain and pooled, with
+    a workspace and without) and one on position rows for each where staging them could pay; nothing is left
+    for the forward itself, nor where its result is pooled."""
+    for c, h, w, most in ((64, 54, 47, 8), (256, 15, 13, 8), (3, 9, 20, 4)):
+        layer, x = make(c, c, h, w)
+        sizes = made(lambda: (layer.workspace(x.shape), layer.scratch(x.shape)))
+        assert 0 < sizes <= most, (c, h, w, sizes)
+        for pool in (False, True):
+            assert made(lambda: layer.forward(x, split=True, pool=pool)) == 0, (c, h, w)
+            assert made(lambda: layer.forward(x, pool=pool)) == 0, (c, h, w)
+        layer.close()
+
+
+def test_a_stack_with_a_pinned_kernel_plans_nothing():
+    layers = [make(24, 40, 23, 21)[0], make(40, 16, 23, 21)[0]]
+    for flags in (B.KERNEL_TILED, B.KERNEL_SIMPLE, B.ROWS4):
+        assert made(lambda: B.Stack(layers, [False, True], 1, 23, 21, B.RELU | flags)) == 0
+    assert made(lambda: B.Stack(layers, [False, True], 1, 23, 21, B.RELU)) > 0
+    for l in layers:
+        l.close()
