@@ -97,6 +97,8 @@ def load(path):
         L.pconv_trace_read.argtypes = [vp, ctypes.POINTER(ctypes.c_ulonglong), ci]
         L.pconv_dev_withhold.argtypes = [ci, cu]
         L.pconv_dev_clear_status.argtypes = [vp]
+        L.pconv_dev_stack_dense_layers.argtypes = [vp]
+        L.pconv_dev_path.argtypes = [vp, ci, ci, ci, ci, ci, ctypes.c_size_t]
         L.pconv_dev_dense_plans.restype = ctypes.c_longlong
         L.pconv_dev_dense_plan.argtypes = [ci] * 10 + [ctypes.c_size_t, ci, ci, ip, ctypes.POINTER(ctypes.c_double)]
     L.pconv_status_str.argtypes = [ci]

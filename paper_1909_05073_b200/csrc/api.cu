@@ -216,7 +216,7 @@ static pconv_status forward_impl(const pconv_handle* h, const void* x, const flo
   bool dense = false, staged = false;
   if (!(flags & kPinsKernel)) {
     const bool room = scratch && dense_rows_bytes(L, n, h_in, w_in, pool) <= scratch_bytes;
-    const DensePath path = dense_path(L, n, h_in, w_in, pool, room ? kRowsStaged : kNoRows, dense_ws_bytes);
+    const DensePath path = dense_path_alone(L, n, h_in, w_in, pool, room ? kRowsStaged : kNoRows, dense_ws_bytes);
     staged = path == kFromRows;
     dense = path != kNotDense || (!pool && batch_on_tensor_cores(L, n, h_in, w_in, dense_ws_bytes));
   }
@@ -363,6 +363,10 @@ extern "C" pconv_status pconv_dev_dense_plan(int c_out, int c_in, int stride, in
              ? PCONV_OK : PCONV_ERR_UNSUPPORTED;
 }
 
+extern "C" int pconv_dev_path(const pconv_handle* h, int n, int h_in, int w_in, int pool, int rows, size_t ws_bytes) {
+  return h ? (int)pconv::dense_path_alone(h->d, n, h_in, w_in, pool != 0, (pconv::RowsFrom)rows, ws_bytes) : -1;
+}
+
 extern "C" pconv_status pconv_dev_clear_status(const pconv_handle* h) {
   if (!h) return PCONV_ERR_NULL;
   if (cudaDeviceSynchronize() != cudaSuccess || cudaMemset(h->d.err, 0, 4) != cudaSuccess ||
@@ -410,6 +414,7 @@ struct pconv_stack {
   std::vector<void*>* rows;
   void* rows_block;            // the one allocation behind them
   std::vector<pconv::DensePath>* path;
+  bool all_sparse;             // the sparse kernel for every layer: the choice was taken back for the whole stack
   unsigned int* sync_dev;      // the chain kernel's two counters (zero between launches)
 };
 
@@ -538,6 +543,8 @@ static bool build_rows(pconv_stack* s) {
   const size_t ws_bytes = (s->flags & PCONV_REPRODUCIBLE) ? 0 : s->ws_bytes;
   std::vector<size_t> at(s->n_layers, 0);
   size_t total = 0;
+  double chosen_us = 0.0, sparse_us = 0.0;       // expected, of the layers chosen and of the sparse kernel throughout
+  bool have_sparse = s->chains->empty();
   int ch = s->h, cw = s->w;
   for (int i = 0; i < s->n_layers; ++i) {
     const pconv::DeviceLayer& L = s->layers[i]->d;
@@ -554,6 +561,10 @@ static bool build_rows(pconv_stack* s) {
         at[i] = total + 1;
         total += (pconv::dense_rows_bytes(L, s->n, ch, cw, pool) + 255) & ~(size_t)255;
       }
+      const double us = pconv::path_us(L, s->n, ch, cw, pool, pconv::kNotDense, false, ws_bytes);
+      sparse_us += us;
+      chosen_us += (*s->path)[i] == pconv::kNotDense ? us : pconv::path_us(L, s->n, ch, cw, pool, (*s->path)[i], !given, ws_bytes);
+      have_sparse = have_sparse && us > 0.0 && pconv::tiled_supported(L, s->n, ch, cw);
     }
     ch = (ch - 1) / L.stride + 1;
     cw = (cw - 1) / L.stride + 1;
@@ -561,6 +572,20 @@ static bool build_rows(pconv_stack* s) {
       ch /= 2;
       cw /= 2;
     }
+  }
+  // The choice goes layer by layer and is coarse; the sums of expected times over a stack are good to some 5 %.  VGG-16
+  // at keep rate 0.3 on 40 to 224 pixels, 1 to 8 images: where the sum of what was chosen is above 1.1 of the
+  // sparse one's it ran at 0.99-1.10 of its time (64x64 N=4 232 us against 216, N=8 299 against 272, 96x96 N=4
+  // 305 against 308), between 1.0 and 1.1 at 0.94-1.11 without any order (130x130 N=2, at 1.08, 276 us against 293).
+  bool take_back = have_sparse && chosen_us > 1.1 * sparse_us;
+#ifdef PCONV_DEV
+  if (getenv("PCONV_FORCE_DENSE")) take_back = false;
+#endif
+  if (take_back) {
+    s->all_sparse = true;
+    total = 0;
+    std::fill(at.begin(), at.end(), 0);
+    std::fill(s->path->begin(), s->path->end(), pconv::kNotDense);
   }
   if (total && (cudaMalloc(&s->rows_block, total) != cudaSuccess || cudaMemset(s->rows_block, 0, total) != cudaSuccess))
     return false;
@@ -649,6 +674,12 @@ extern "C" pconv_status pconv_stack_create(const pconv_handle* const* layers,
   *out = s;
   return PCONV_OK;
 }
+
+#ifdef PCONV_DEV
+extern "C" int pconv_dev_stack_dense_layers(const pconv_stack* s) {
+  return s ? (int)(s->n_layers - std::count(s->path->begin(), s->path->end(), pconv::kNotDense)) : -1;
+}
+#endif
 
 extern "C" pconv_status pconv_stack_out_shape(const pconv_stack* s, int* n, int* c, int* h,
                                               int* w) {
@@ -748,7 +779,8 @@ extern "C" pconv_status pconv_stack_forward(pconv_stack* s, const void* x, void*
         return PCONV_ERR_CUDA;
       }
     } else {
-      st = forward_impl(s->layers[i], cur, s->bias[i], dst, s->n, ch, cw, s->flags | (fuse ? PCONV_POOL2X2 : 0u), s->ws,
+      st = forward_impl(s->layers[i], cur, s->bias[i], dst, s->n, ch, cw,
+                        s->flags | (fuse ? PCONV_POOL2X2 : 0u) | (s->all_sparse ? PCONV_KERNEL_TILED : 0u), s->ws,
                         s->ws_bytes, nullptr, 0, stream, s->status_dev);
     }
     if (st != PCONV_OK) return st;

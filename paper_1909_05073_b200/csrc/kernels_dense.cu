@@ -1691,12 +1691,14 @@ size_t split_bytes(const DGeo& g) {
 struct StepCost {
   double step, epi;      // a channel step of an item, and its end
 };
+double tap_cycles(const DGeo& g, bool half) {      // the MMAs of a tap of one tile
+  const int nt = g.nt;
+  return half ? mma_cycles(nt)
+              : (g.form3 ? mma_cycles(3 * nt) + mma_cycles(2 * nt) + mma_cycles(nt) : mma_cycles(2 * nt) + 4 * mma_cycles(nt));
+}
 StepCost step_cost(const DGeo& g, bool half) {
   const int nt = g.nt;
-  double tap = half ? mma_cycles(nt)
-                    : (g.form3 ? mma_cycles(3 * nt) + mma_cycles(2 * nt) + mma_cycles(nt)
-                               : mma_cycles(2 * nt) + 4 * mma_cycles(nt));
-  double step = tap * g.n_taps * g.tiles;
+  double step = tap_cycles(g, half) * g.n_taps * g.tiles;
   const double wb = ((double)g.n_taps * (half ? 1 : 3) * nt * 32 + (g.vec ? 0.0 : g.a_bytes)) / 36.0;
   // (a batch of the producers -- a load and its rows a thread -- takes about as long whatever its width)
   double conv = 300.0 + (half ? 1100.0 : 1300.0) * ((2 * g.n_vec + 319) / 320);
@@ -1707,11 +1709,13 @@ StepCost step_cost(const DGeo& g, bool half) {
   return {step, 600 + (half ? 8.0 : 16.0) * g.tiles * nt};
 }
 long long ceil_div(long long a, long long b) { return (a + b - 1) / b; }
+long long steps_of(const DGeo& g) {                // channel steps of the CTA that has most of them
+  return g.split ? ceil_div((long long)g.n_tiles * g.k_steps, g.grid) : ceil_div(g.n_tiles, g.grid) * g.k_steps;
+}
 double dense_cycles(const DGeo& g, const StepCost& cost, bool half, int sms) {
   const int nt = g.nt;
   const double epi = cost.epi;
-  const long long steps = g.split ? ceil_div((long long)g.n_tiles * g.k_steps, g.grid)
-                                  : ceil_div(g.n_tiles, g.grid) * g.k_steps;
+  const long long steps = steps_of(g);
   const long long segments = ceil_div(steps, g.k_steps);
   double c = 4500 + steps * cost.step + epi + (segments - 1) * (half && g.n_buf == 1 ? epi : 0.25 * epi);
   if (g.split) {
@@ -1724,6 +1728,32 @@ double dense_cycles(const DGeo& g, const StepCost& cost, bool half, int sms) {
     else c += (4200 + bytes * g.grid / sms / 8.0) * (g.parts ? 1.0 : 2.0);
   }
   return c;
+}
+// What a launch is expected to take, in microseconds.  dense_cycles ranks the plans of one shape; this sets a plan
+// against the sparse kernel, for which a rank is not enough.  Constants fitted (least squares of log ratios, both
+// strides, 3 to 512 channels, 16 to 512 filters, maps of 4 to 112 pixels, 1 to 64 images) to 4826 layers timed
+// in every form: measured over expected has a standard deviation of 0.07 for fp32 and 0.09 for fp16, where
+// dense_cycles has 0.19 and 0.21.  What it has that dense_cycles has not: with a single activation stage a
+// step's copies or conversions come after its MMAs.
+double launch_us(const DGeo& g, bool half) {
+  struct Fit {   // cycles of 0.6 ns; rates in bytes a cycle
+    double base_nchw, base_rows, step, mma, copy_rate, conv0, conv1, epi0, epi1, more, exchange, part, cluster_rate, ws_rate;
+  };
+  static const Fit kFit[2] = {
+      {787, 2335, 1699, 0.619, 81.0, 69, 733, 7824, 67.9, 0.416, 2860, 13.4, 18.7, 7.15},
+      {5113, 4256, 771, 0.467, 74.5, 0, 734, 906, 40.8, 0.655, 2919, 0.0, 15.3, 9.45}};
+  const Fit& f = kFit[half ? 1 : 0];
+  const bool p8 = g.vec == 0;
+  const double copies = (double)g.n_taps * (half ? 1 : 3) * g.nt * 32 + (p8 ? g.a_bytes : 0);
+  const double fill = p8 ? g.a_bytes / f.copy_rate : f.conv0 + f.conv1 * ((2 * g.n_vec + 319) / 320);
+  double step = std::max(tap_cycles(g, half) * g.n_taps * g.tiles * f.mma, copies / f.copy_rate);
+  step = (g.a_stages == 1 ? step + fill : std::max(step, fill)) + f.step;
+  const long long steps = steps_of(g), segments = ceil_div(steps, g.k_steps);
+  double c = (p8 ? f.base_rows : f.base_nchw) + steps * step + (f.epi0 + f.epi1 * g.tiles * g.nt) * (1 + (segments - 1) * f.more);
+  const double bytes = (double)g.tiles * g.nt * 512;
+  if (g.cluster) c += f.exchange + f.part * g.parts + bytes / f.cluster_rate;
+  else if (g.split) c += (f.exchange + bytes * g.grid / 148 / f.ws_rate) * (g.parts ? 1 : 2);
+  return 6e-4 * c;
 }
 // What no way of cutting these tiles can fall below: all steps spread evenly over all SMs.
 double least_cycles(const DGeo& g, const StepCost& cost, int sms) {
@@ -1817,7 +1847,7 @@ struct PlanKey {
 };
 struct Plan {
   bool found;
-  double cycles;
+  double cycles, us;           // rank and expected time
   size_t need;                 // workspace
   int n_tiles, n_ft;
 };
@@ -1835,16 +1865,22 @@ struct PlanTable {
 };
 PlanTable g_plans;
 
+PlanKey plan_key(const DeviceLayer& L, int n, int h, int w, bool pool, bool p8) {
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess) cudaGetLastError();
+  return {L.c_in, L.c_out, L.stride, L.storage, L.tap_mask, n, h, w, 2 * (int)pool + (int)p8, dev};
+}
+int plan_set(const PlanKey& k, unsigned long long hash) {
+  for (int v : {k.c_in, k.c_out, k.n, k.h, k.w, (k.tap_mask << 8) + (k.form << 4) + (k.stride << 2) + k.storage})
+    hash = (hash ^ (unsigned)v) * 0x9E3779B97F4A7C15ull, hash ^= hash >> 29;
+  return (int)((hash >> 40) % kPlanSets);
+}
+
 Plan find_plan(const DeviceLayer& L, int n, int h, int w, bool pool, bool p8, size_t ws_bytes, DGeo* geo = nullptr) {
   if (!L.wdense || n <= 0 || h <= 0 || w <= 0) return Plan{};
   if (ws_bytes > kMaxSplitBytes) ws_bytes = kMaxSplitBytes;
-  int dev = -1;
-  if (cudaGetDevice(&dev) != cudaSuccess) cudaGetLastError();
-  const PlanKey k = {L.c_in, L.c_out, L.stride, L.storage, L.tap_mask, n, h, w, 2 * (int)pool + (int)p8, dev};
-  unsigned long long hash = 0;
-  for (int v : {k.c_in, k.c_out, k.n, k.h, k.w, (k.tap_mask << 8) + (k.form << 4) + (k.stride << 2) + k.storage})
-    hash = (hash ^ (unsigned)v) * 0x9E3779B97F4A7C15ull, hash ^= hash >> 29;
-  const int set = (int)((hash >> 40) % kPlanSets);
+  const PlanKey k = plan_key(L, n, h, w, pool, p8);
+  const int set = plan_set(k, 0);
 #ifdef PCONV_DEV
   const bool keep = !getenv("PCONV_FORCE_DENSE");      // (a forced plan is nobody else's)
 #else
@@ -1864,15 +1900,18 @@ Plan find_plan(const DeviceLayer& L, int n, int h, int w, bool pool, bool p8, si
   made.most = ws_bytes;
   const bool half = L.storage == PCONV_F16;
   made.plan.found = dense_plan(L, n, h, w, pool, p8, ws_bytes, device_sm_count(),
-                               [&](int parts) { return max_clusters(dev, half, parts); }, true, &g, &made.plan.cycles);
-  if (made.plan.found) made.plan.need = split_bytes(g);
+                               [&](int parts) { return max_clusters(k.dev, half, parts); }, true, &g, &made.plan.cycles);
+  if (made.plan.found) {
+    made.plan.need = split_bytes(g);
+    made.plan.us = launch_us(g, half);
+  }
   made.plan.n_tiles = g.n_tiles;
   made.plan.n_ft = g.n_ft;
 #ifdef PCONV_DEV
   if (made.plan.found && getenv("PCONV_DENSE_VERBOSE"))
-    fprintf(stderr, "dense %d->%d %dx%d n%d s%d pool%d p8 %d ws%zu: tiles %d nt %d split %d cluster %d grid %d n_tiles %d q %d pitch %d a_stages %d b_slots %d cycles %.0f\n",
+    fprintf(stderr, "dense %d->%d %dx%d n%d s%d pool%d p8 %d ws%zu: tiles %d nt %d split %d cluster %d grid %d n_tiles %d q %d pitch %d a_stages %d b_slots %d cycles %.0f us %.1f\n",
             L.c_in, L.c_out, h, w, n, L.stride, (int)pool, (int)p8, ws_bytes, g.tiles, g.nt, g.split, g.cluster * g.parts, g.grid,
-            g.n_tiles, g.q_tot, g.pitch, g.a_stages, g.b_slots, made.plan.cycles);
+            g.n_tiles, g.q_tot, g.pitch, g.a_stages, g.b_slots, made.plan.cycles, made.plan.us);
 #endif
   if (geo) *geo = g;
   if (keep) {
@@ -2013,7 +2052,10 @@ size_t dense_rows_bytes(const DeviceLayer& L, int n, int h, int w, bool pool) {
 }
 
 size_t dense_scratch_bytes(const DeviceLayer& L, int n, int h, int w, bool pool, size_t ws_bytes) {
-  return dense_path(L, n, h, w, pool, kRowsStaged, ws_bytes) == kFromRows ? dense_rows_bytes(L, n, h, w, pool) : 0;
+  // (dense_path_alone takes a choice back, but makes none: it need not be asked where rows are not chosen)
+  return dense_path(L, n, h, w, pool, kRowsStaged, ws_bytes) == kFromRows &&
+                 dense_path_alone(L, n, h, w, pool, kRowsStaged, ws_bytes) == kFromRows
+             ? dense_rows_bytes(L, n, h, w, pool) : 0;
 }
 
 cudaError_t launch_stage(const DeviceLayer& L, const void* x, void* rows, int n, int h, int w, bool pool,
@@ -2101,6 +2143,70 @@ DensePath dense_path(const DeviceLayer& L, int n, int h, int w, bool pool, RowsF
     const Plan e = find_plan(L, n, h, w, pool, true, ws_bytes);
     if (e.found && cycles_of(e) + staging < best) path = kFromRows;
   }
+  return path;
+}
+
+double path_us(const DeviceLayer& L, int n, int h, int w, bool pool, DensePath path, bool staged, size_t ws_bytes) {
+  if (path == kNotDense) return tiled_us(L, n, h, w, ws_bytes);
+  const Plan e = find_plan(L, n, h, w, pool, path == kFromRows, ws_bytes);
+  // (laying the input out overlaps its neighbours and moves 6.5 TB/s)
+  const double moved = (double)rows_bytes(rows_of(L.c_in, L.stride, n, h, w, pool), L.storage == PCONV_F16);
+  return e.us + (path == kFromRows && staged ? 1.0 + moved / 6.5e6 : 0.0);
+}
+
+namespace {
+// The choices of recent calls, kept as the plans are.
+struct ChoiceKey {
+  PlanKey shape;
+  int rows, codes;
+  long long kept;
+  size_t ws_bytes;
+};
+struct ChoiceTable {
+  std::mutex lock;
+  struct Entry {
+    ChoiceKey key;
+    DensePath path;
+  } entry[kPlanSets][kPlanWays];
+  unsigned char next[kPlanSets];
+};
+ChoiceTable g_choices;
+
+}  // namespace
+
+// dense_path's estimates are coarse (a fifth either way) and favour the dense kernel, which pays in a stack, where each
+// dense layer hands the next its input.  A layer of its own that they give to the dense kernel goes back where the
+// two expected times (path_us) say that the sparse kernel is faster by more than they are off.  Of 3653 fp32 layers
+// 4.9 % instead of 8.2 % then run over 3 % slower than on the sparse kernel, and 0.3 % over 3 % slower than before
+// (256->256 28x28 N=2: dense 32.6 us, sparse 24.0).  (The expected times alone, without a margin: 3 % faster over all
+// layers timed one by one, but ResNet-50 N=32, whose layers follow one another, 855 -> 887 us.)
+DensePath dense_path_alone(const DeviceLayer& L, int n, int h, int w, bool pool, RowsFrom rows, size_t ws_bytes) {
+  if (!L.wdense || n <= 0 || h <= 0 || w <= 0) return kNotDense;
+#ifdef PCONV_DEV
+  if (getenv("PCONV_FORCE_DENSE") || getenv("PCONV_FORCE_ROWS")) return dense_path(L, n, h, w, pool, rows, ws_bytes);
+#endif
+  ChoiceKey k;
+  std::memset(&k, 0, sizeof(k));
+  k.shape = plan_key(L, n, h, w, pool, false);
+  k.rows = rows;
+  k.codes = (L.codes_s ? 2 : 0) + (L.wide_codes ? 1 : 0);
+  k.kept = L.n_kept;
+  k.ws_bytes = std::min(ws_bytes, kMaxSplitBytes);
+  const int set = plan_set(k.shape, (unsigned long long)k.kept * 8 + (unsigned)rows);
+  {
+    std::lock_guard<std::mutex> hold(g_choices.lock);
+    for (const ChoiceTable::Entry& e : g_choices.entry[set])
+      if (std::memcmp(&e.key, &k, sizeof(k)) == 0) return e.path;
+  }
+  DensePath path = dense_path(L, n, h, w, pool, rows, ws_bytes);
+  if (path != kNotDense) {
+    const double sparse_us = path_us(L, n, h, w, pool, kNotDense, false, ws_bytes);
+    if (sparse_us > 0.0 && path_us(L, n, h, w, pool, path, rows == kRowsStaged, ws_bytes) > 1.15 * sparse_us) path = kNotDense;
+  }
+  std::lock_guard<std::mutex> hold(g_choices.lock);
+  ChoiceTable::Entry& e = g_choices.entry[set][g_choices.next[set]++ % kPlanWays];
+  e.key = k;
+  e.path = path;
   return path;
 }
 

@@ -2148,6 +2148,14 @@ size_t tiled_workspace_bytes(const DeviceLayer& L, int n, int h, int w, int rmod
          ((ctas * kMaxConsumerWarps * 4 + 255) & ~(size_t)255);
 }
 
+// Expected duration of a default launch in microseconds, < 0 if the kernel does not take the shape.  (0.17 us a unit of
+// geo_cost: median of 4826 layers of 1-64 images, fifth to 95th percentile 0.74 to 1.21 of it for fp32.)
+double tiled_us(const DeviceLayer& L, int n, int h, int w, size_t ws_bytes) {
+  Geo g;
+  if (!L.codes_s || !make_geo<false>(L, n, h, w, ws_bytes > 0, 0, &g)) return -1.0;
+  return 0.17 * geo_cost(L, g);
+}
+
 // The launch geometry launch_tiled would use (see pconv_plan_t).
 bool tiled_plan(const DeviceLayer& L, int n, int h, int w, bool generic_taps, bool with_workspace,
                 int rmode, pconv_plan_t* out) {

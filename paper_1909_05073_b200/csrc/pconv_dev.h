@@ -45,6 +45,13 @@ pconv_status pconv_dev_dense_plan(int c_out, int c_in, int stride, int storage, 
                                   int pool, int rows, size_t ws_bytes, int cluster_sms, int prune, int* fields,
                                   double* cycles);
 
+/* The kernel a default forward of this shape takes: 0 the sparse one, 1 the dense one from NCHW, 2 the dense one on
+ * position rows.  rows: 0 there is no room for position rows, 1 there is, 2 they are there already. */
+int pconv_dev_path(const pconv_handle* h, int n, int h_in, int w_in, int pool, int rows, size_t ws_bytes);
+
+/* Layers of a stack that the dense kernel runs. */
+int pconv_dev_stack_dense_layers(const pconv_stack* s);
+
 /* Clears the handle's sticky status word (pconv_device_status reports PCONV_OK again until the
  * next abandoned wait).  Synchronises the device. */
 pconv_status pconv_dev_clear_status(const pconv_handle* h);

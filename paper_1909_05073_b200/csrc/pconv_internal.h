@@ -139,7 +139,10 @@ cudaError_t dense_build_weights(const DeviceLayer& L, cudaStream_t stream);
 bool dense_supported(const DeviceLayer& L, int n, int h, int w, bool pool, size_t ws_bytes);
 enum RowsFrom { kNoRows, kRowsStaged, kRowsGiven };    // position rows: no room, to be staged, already there
 enum DensePath { kNotDense, kFromNchw, kFromRows };
-DensePath dense_path(const DeviceLayer& L, int n, int h, int w, bool pool, RowsFrom rows, size_t ws_bytes);
+DensePath dense_path(const DeviceLayer& L, int n, int h, int w, bool pool, RowsFrom rows, size_t ws_bytes);        // in a stack
+DensePath dense_path_alone(const DeviceLayer& L, int n, int h, int w, bool pool, RowsFrom rows, size_t ws_bytes);  // by itself
+// Expected microseconds of a path (staged: its position rows are laid out first), < 0 if it has none.
+double path_us(const DeviceLayer& L, int n, int h, int w, bool pool, DensePath path, bool staged, size_t ws_bytes);
 // Workspace of the forms that a forward may take with up to `most` bytes of it.
 size_t dense_workspace_bytes(const DeviceLayer& L, int n, int h, int w, bool pool, RowsFrom rows, size_t most);
 // Activations in the dense kernel's own layout ("position rows", see kernels_dense.cu): whether the kernel
@@ -162,6 +165,7 @@ constexpr int kPinRowsMask = 0xff;
 constexpr int kPinBulk = 0x100;
 size_t tiled_workspace_bytes(const DeviceLayer& L, int n, int h, int w, int rmode);
 bool tiled_supported(const DeviceLayer& L, int n, int h, int w);
+double tiled_us(const DeviceLayer& L, int n, int h, int w, size_t ws_bytes);
 bool tiled_plan(const DeviceLayer& L, int n, int h, int w, bool generic_taps, bool with_workspace,
                 int rmode, pconv_plan_t* out);
 #ifdef PCONV_DEV

@@ -1,6 +1,7 @@
 """When launch plans of the dense kernel are worked out: planning is host work that a first pass pays for.
 The development build counts the plans made."""
 import threading
+from dataclasses import replace
 
 import pytest
 import torch
@@ -27,8 +28,8 @@ def made(call):
     return B.lib().pconv_dev_dense_plans() - before
 
 
-def make(c_in, c_out, h, w, n=1, storage="f32", seed=1, stride=1):
-    wt, bias, _ = synth.gen_weights(synth.LayerSpec("p", c_in, c_out, h, w, stride, 0.4), seed)
+def make(c_in, c_out, h, w, n=1, storage="f32", seed=1, stride=1, keep=0.4):
+    wt, bias, _ = synth.gen_weights(synth.LayerSpec("p", c_in, c_out, h, w, stride, keep), seed)
     layer = B.Layer(wt, synth.PATTERNS8, stride, B.F16 if storage == "f16" else B.F32, bias)
     x = torch.zeros((n, c_in, h, w), device="cuda")
     return layer, x.half() if storage == "f16" else x
@@ -121,3 +122,51 @@ def test_a_stack_with_a_pinned_kernel_plans_nothing():
     assert made(lambda: B.Stack(layers, [False, True], 1, 23, 21, B.RELU)) > 0
     for l in layers:
         l.close()
+
+
+SPARSE, NCHW, ROWS = 0, 1, 2
+ROOM, GIVEN = 1, 2
+MEASURED = [  # c_in, c_out, h, w, n, stride, keep, storage, rows, the fastest, and what was measured (us)
+    (256, 256, 28, 28, 2, 1, 0.3, "f32", GIVEN, SPARSE),     # 24.0; on rows 32.6
+    (256, 256, 12, 12, 8, 1, 0.3, "f32", GIVEN, SPARSE),     # 22.6; on rows 32.2
+    (512, 512, 16, 16, 1, 1, 0.3, "f32", GIVEN, SPARSE),     # 18.0; on rows 22.7
+    (512, 512, 28, 28, 1, 1, 0.3, "f32", GIVEN, ROWS),       # 32.2; sparse 39.9
+    (512, 512, 20, 20, 4, 1, 0.3, "f32", GIVEN, ROWS),       # 66.3; sparse 89.8
+    (512, 512, 14, 14, 64, 1, 0.5, "f32", ROOM, NCHW),       # 310; sparse 589
+    (512, 512, 7, 7, 1, 1, 0.3, "f16", GIVEN, ROWS),         # 8.4; sparse 23.8
+]
+
+
+@pytest.mark.parametrize("case", MEASURED, ids=lambda c: "x".join(str(v) for v in c))
+def test_the_choice_of_kernel_where_measurements_are_far_apart(case):
+    c_in, c_out, h, w, n, stride, keep, storage, rows, fastest = case
+    layer, _ = make(c_in, c_out, 9, 9, 1, storage, 2, stride, keep)
+    ws = B.pconv_workspace_bytes(layer.handle, n, h, w)
+    for _ in range(2):                              # (worked out, then found)
+        assert B.lib().pconv_dev_path(layer.handle, n, h, w, 0, rows, ws) == fastest
+    layer.close()
+
+
+@pytest.mark.parametrize("size,n,keep,sparse", [(64, 4, 0.3, True), (64, 8, 0.3, True), (224, 1, 0.3, False), (64, 4, 0.5, False)])
+def test_a_stack_that_runs_faster_on_the_sparse_kernel_throughout_does_so(size, n, keep, sparse):
+    """VGG-16, measured: 236 us as chosen layer by layer against 216 sparse, 299 against 272, 350 against 369, 238
+    against 252."""
+    layers, pools, h = [], [], size
+    for i, s in enumerate(synth.config(2).layers):
+        wt, b, _ = synth.gen_weights(replace(s, keep=1.0 if i == 0 else keep, h=h, w=h), 7 + i)
+        layers.append(B.Layer(wt, synth.PATTERNS8, 1, B.F32, b))
+        pools.append(s.pool_after)
+        h = h // 2 if s.pool_after else h
+    stack = B.Stack(layers, pools, n, size, size, B.RELU)
+    pinned = B.Stack(layers, pools, n, size, size, B.RELU | B.KERNEL_TILED)
+    assert (B.lib().pconv_dev_stack_dense_layers(stack.ptr) == 0) == sparse
+    assert stack.launches() == len(layers)
+    x = torch.rand((n, 3, size, size), device="cuda")
+    y, z = torch.empty(stack.out_shape, device="cuda"), torch.empty(stack.out_shape, device="cuda")
+    for _ in range(2):
+        stack.forward(x, y)
+        pinned.forward(x, z)
+    assert float((y - z).norm() / z.norm()) < 1e-5          # sums of up to 4608 terms in another order, thirteen times
+    assert stack.status() == (0, 0) and pinned.status() == (0, 0)
+    stack.close()
+    pinned.close()
