@@ -76,6 +76,8 @@ constexpr int kHeader = 1024;             // barriers, Tensor Memory address, bi
 constexpr int kBiasOff = 512;
 static_assert(16 * (kMaxA + kMaxB) + 32 + 4 + 16 <= kBiasOff, "barriers, Tensor Memory address, segments to redo");
 constexpr uint32_t kSpinLimit = 1u << 20;
+// Wait ids in the status word (the tiled kernel's are below 20): a free stage or slot, a filled one, accumulators.
+constexpr int kWaitFree = 21, kWaitFull = 22, kWaitSums = 23;
 constexpr uint32_t kWaitHintNs = 200;
 constexpr int kSmemLimit = 227 * 1024;
 constexpr int kTables = 5;                // load tables of the NCHW producers: segments s - 1 .. s + 3
@@ -809,15 +811,15 @@ __device__ __forceinline__ void mma_role(const DeviceLayer& L, const DGeo& g, ui
     for (int seg = 0; get_item(g, share, seg, &it); ++seg) {
       if constexpr (HALF) {
         const uint32_t buf = g.n_buf == 2 ? (sc & 1u) : 0u, use = g.n_buf == 2 ? sc >> 1 : sc;
-        wait(bar.ce + 8 * buf, (use & 1u) ^ 1u, 3, 1);
+        wait(bar.ce + 8 * buf, (use & 1u) ^ 1u, kWaitSums, 1);
         const uint32_t d0 = tmem + buf * 256u;
         for (int ks = it.k0; ks < it.k1; ++ks) {
-          wait(bar.af + 8 * sa, pa, 2, 2);
+          wait(bar.af + 8 * sa, pa, kWaitFull, 2);
           const u64 a_st = a_d0 + ((sdesc + (uint32_t)g.a_off + (uint32_t)sa * (uint32_t)g.a_bytes) >> 4);
 #pragma unroll
           for (int t = 0; t < 9; t += 3) {                 // three taps to a slot
             if (t >= g.n_taps) break;
-            wait(bar.bf + 8 * sb, pb, 2, 3);
+            wait(bar.bf + 8 * sb, pb, kWaitFull, 3);
             const u64 b_t = slot_desc(sb);
 #pragma unroll
             for (int v = 0; v < 3; ++v) {
@@ -841,8 +843,8 @@ __device__ __forceinline__ void mma_role(const DeviceLayer& L, const DGeo& g, ui
         // of the last step -- their main products, then the other taps.
         for (int ks = it.k0; ks < it.k1; ++ks, ++sc) {
           const bool first = ks == it.k0;
-          if (first) wait(bar.ce, (sc & 1u) ^ 1u, 3, 1);
-          wait(bar.af + 8 * sa, pa, 2, 2);
+          if (first) wait(bar.ce, (sc & 1u) ^ 1u, kWaitSums, 1);
+          wait(bar.af + 8 * sa, pa, kWaitFull, 2);
           const u64 a_st = a_d0 + ((sdesc + (uint32_t)g.a_off + (uint32_t)sa * (uint32_t)g.a_bytes) >> 4);
           auto cross = [&](int j, int t, u64 b_t) {
             const u64 a1 = a_st + (uint32_t)g.tap_off[j][t], a2 = a1 + slab, a3 = a2 + slab;
@@ -873,17 +875,17 @@ __device__ __forceinline__ void mma_role(const DeviceLayer& L, const DGeo& g, ui
 #pragma unroll
           for (int t = 0; t < kPre; ++t) {
             if (t >= g.n_taps) break;
-            wait(bar.bf + 8 * s2, p2, 2, 3);
+            wait(bar.bf + 8 * s2, p2, kWaitFull, 3);
             const u64 b_t = slot_desc(s2);
 #pragma unroll
             for (int j = 0; j < TILES; ++j) cross(j, t, b_t);
             if (++s2 == g.b_slots) { s2 = 0; p2 ^= 1; }
           }
-          if (!first) wait(bar.ce, (sc & 1u) ^ 1u, 3, 1);
+          if (!first) wait(bar.ce, (sc & 1u) ^ 1u, kWaitSums, 1);
 #pragma unroll
           for (int t = 0; t < 9; ++t) {
             if (t >= g.n_taps) break;
-            if (t >= kPre) wait(bar.bf + 8 * sb, pb, 2, 3);
+            if (t >= kPre) wait(bar.bf + 8 * sb, pb, kWaitFull, 3);
             const u64 b_t = slot_desc(sb);
 #pragma unroll
             for (int j = 0; j < TILES; ++j) {
@@ -930,7 +932,7 @@ __device__ __forceinline__ void weight_role(const DeviceLayer& L, const DGeo& g,
         const uint32_t slot_bar = bar.bf + 8 * sb;
         const long long t_ = T_NOW();
         if (!mbar_test(bar.be + 8 * sb, (uint32_t)(pb ^ 1)))
-          if (!failed) failed = !warp_wait(bar.be + 8 * sb, (uint32_t)(pb ^ 1), L.err, 1);
+          if (!failed) failed = !warp_wait(bar.be + 8 * sb, (uint32_t)(pb ^ 1), L.err, kWaitFree);
         T_ADD(6, t_);
         const uint32_t dst = sbase + (uint32_t)g.b_off + (uint32_t)sb * (uint32_t)g.b_bytes;
         if (failed) break;
@@ -955,7 +957,7 @@ __device__ __forceinline__ void weight_role(const DeviceLayer& L, const DGeo& g,
   // no copy is in flight when the CTA ends, whatever made it end
   for (int s = 0; s < g.b_slots; ++s) {
     if (s >= sb && !wrapped) break;
-    warp_wait(bar.bf + 8 * s, (uint32_t)(s < sb ? pb : pb ^ 1), L.err, 2);
+    warp_wait(bar.bf + 8 * s, (uint32_t)(s < sb ? pb : pb ^ 1), L.err, kWaitFull);
   }
   if (lane == 0) T_FLUSH(6, 6);
 }
@@ -982,7 +984,7 @@ __device__ __forceinline__ void activation_role(const DeviceLayer& L, const DGeo
     for (int ks = it.k0; ks < it.k1; ++ks) {
       const long long t_ = T_NOW();
       if (!mbar_test(bar.ae + 8 * sa, (uint32_t)(pa ^ 1)))
-        if (!failed) failed = !warp_wait(bar.ae + 8 * sa, (uint32_t)(pa ^ 1), L.err, 1);
+        if (!failed) failed = !warp_wait(bar.ae + 8 * sa, (uint32_t)(pa ^ 1), L.err, kWaitFree);
       T_ADD(5, t_);
       if (failed || ks - it.k0 == withhold) break;
       const uint32_t full = bar.af + 8 * sa;
@@ -1004,7 +1006,7 @@ __device__ __forceinline__ void activation_role(const DeviceLayer& L, const DGeo
   // no copy is in flight when the CTA ends, whatever made it end
   for (int s = 0; s < g.a_stages; ++s) {
     if (s >= sa && !wrapped) break;
-    warp_wait(bar.af + 8 * s, (uint32_t)(s < sa ? pa : pa ^ 1), L.err, 2);
+    warp_wait(bar.af + 8 * s, (uint32_t)(s < sa ? pa : pa ^ 1), L.err, kWaitFull);
   }
   if (lane == 0) T_FLUSH(5, 5);
 }
@@ -1160,7 +1162,7 @@ dense_kernel(const __grid_constant__ DeviceLayer L, const __grid_constant__ DGeo
       }
       if (s_t == pt) {
         const long long t_ = T_NOW();
-        ok = ok && mbar_wait(bar_ae + 8 * sa, (uint32_t)(pa ^ 1), L.err, 1);
+        ok = ok && mbar_wait(bar_ae + 8 * sa, (uint32_t)(pa ^ 1), L.err, kWaitFree);
         T_ADD(5, t_);
       }
       if (ok && s_t < n_tasks) {
@@ -1230,7 +1232,7 @@ dense_kernel(const __grid_constant__ DeviceLayer L, const __grid_constant__ DGeo
       if constexpr (HALF) {
         buf = g.n_buf == 2 ? (sc & 1u) : 0u;
         const long long t_ = T_NOW();
-        ok = warp_wait(bar_cf + 8 * buf, (g.n_buf == 2 ? sc >> 1 : sc) & 1u, L.err, 3);
+        ok = warp_wait(bar_cf + 8 * buf, (g.n_buf == 2 ? sc >> 1 : sc) & 1u, L.err, kWaitSums);
         T_ADD(7, t_);
         ++sc;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -1255,7 +1257,7 @@ dense_kernel(const __grid_constant__ DeviceLayer L, const __grid_constant__ DGeo
         // main sums of every channel step: Tensor Memory -> fp32 registers
         for (int ks = it.k0; ks < it.k1 && ok; ++ks, ++sc) {
           const long long t_ = T_NOW();
-          ok = warp_wait(bar_cf, sc & 1u, L.err, 3);
+          ok = warp_wait(bar_cf, sc & 1u, L.err, kWaitSums);
           T_ADD(7, t_);
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const long long t_main = T_NOW();
