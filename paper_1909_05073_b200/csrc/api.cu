@@ -1,5 +1,6 @@
 // C ABI entry points: argument checks, kernel selection, layer stacks.
 #include <algorithm>
+#include <atomic>
 #include <cstring>
 #include <cstdlib>
 #include <mutex>
@@ -15,7 +16,7 @@ using namespace pconv;
 
 int pconv::device_sm_count() {
   constexpr int kMaxDev = 64, kDefault = 148;
-  static int cached[kMaxDev] = {0};
+  static std::atomic<int> cached[kMaxDev];
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) {
     cudaGetLastError();

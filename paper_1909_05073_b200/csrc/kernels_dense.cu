@@ -1992,7 +1992,7 @@ int max_clusters(int dev, bool half, int parts) {
 template <bool HALF, int V>
 cudaError_t launch_dense_geo(const DeviceLayer& L, const DGeo& g, const void* x, const float* bias, void* y, float* ws,
                              int* tickets, cudaStream_t stream) {
-  static bool ready[64] = {false};
+  static std::atomic<bool> ready[64];
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
