@@ -98,6 +98,45 @@ def test_largest_and_smallest_finite_values(c_in, c_out, h, w, n, stride, where,
     layer.close()
 
 
+# The six products of pieces that the dense kernel forms for fp32, each as the only place where a term of
+# 2^-18 of the result comes from: 2^-9 is half of a bf16 ulp's half, so 1 + 2^-9 + 2^-18 is cut into these three.
+PIECES = [1 + 2.0 ** -9, 1 + 2.0 ** -18 + 2.0 ** -9]
+
+
+@pytest.mark.parametrize("xv", [1.0] + PIECES)
+@pytest.mark.parametrize("wv", [1.0] + PIECES)
+def test_no_product_of_pieces_is_left_out(xv, wv, dense):
+    """All terms alike: sums of 4 x 20 kept terms of at most 24 bits each.  Leaving x2 w2, x1 w3 or x3 w1 out is an
+    error of 3.8e-6 of the result, x1 w2 or x2 w1 one of 2e-3; the products that are left out are below 2^-26
+    of it here (x2 w3, x3 w2), and eighty additions in fp32, truncated where the tensor core adds, err by at most
+    a twentieth of 2^-18 (measured 1e-7)."""
+    c_in, c_out, h, w = 20, 24, 9, 14
+    wt = np.zeros((c_out, c_in, 3, 3), np.float32)
+    for t in (1, 3, 4, 5):
+        wt[:, :, t // 3, t % 3] = wv
+    x = np.full((2, c_in, h, w), xv, np.float32)
+    layer = B.Layer(wt, synth.PATTERNS8, 1, B.F32, None)
+    got = layer.forward(torch.from_numpy(x).cuda(), relu=False).cpu().numpy().astype(np.float64)
+    ref = oracle.conv3x3(x, wt, None, 1, False).astype(np.float64)
+    assert (np.abs(got - ref) <= 8e-7 * ref).all(), np.abs(got / ref - 1).max()
+    layer.close()
+
+
+@pytest.mark.parametrize("c_in,c_out,h,w,n,stride", [(512, 64, 14, 14, 2, 1), (256, 130, 15, 13, 3, 2), (64, 64, 40, 40, 1, 1)])
+def test_fp32_sums_are_as_close_to_64_bits_as_fp32_ones(c_in, c_out, h, w, n, stride, dense):
+    """Norm of the error over norm of the result.  A product of pieces left out alone adds 6.5e-7 here; fp32
+    sums in any order stay near 1e-7 (the sparse kernel is measured beside it, and allowed the same)."""
+    x, wt, bias = make(c_in, c_out, h, w, n, stride)
+    layer = B.Layer(wt, synth.PATTERNS8, stride, B.F32, bias)
+    xt = torch.from_numpy(x).cuda()
+    ref = torch.nn.functional.conv2d(torch.from_numpy(x).double(), torch.from_numpy(wt).double(), torch.from_numpy(bias).double(),
+                                     stride, 1).numpy()
+    off = {k: np.linalg.norm(layer.forward(xt, relu=False, kernel=k).cpu().numpy() - ref) / np.linalg.norm(ref)
+           for k in (0, B.KERNEL_TILED)}
+    assert off[B.KERNEL_TILED] <= 3e-7 and off[0] <= 3e-7, off
+    layer.close()
+
+
 SPECIAL = [np.inf, -np.inf, np.nan, np.inf]
 CASES = [  # (c_in, c_out, h, w, n, stride): ragged channels and filters, several tiles, strips, parity planes
     (24, 40, 12, 13, 2, 1), (33, 75, 9, 30, 2, 1), (8, 40, 3, 300, 1, 1), (40, 24, 15, 10, 3, 2), (5, 130, 1, 9, 2, 2),

@@ -250,12 +250,15 @@ def test_channel_split_path_matches_the_oracle(case, storage):
     if storage == "f16":
         xt = xt.half()
     assert B.pconv_workspace_bytes(layer.handle, n, h, w) > 0
+    assert B.pconv_plan(layer.handle, n, h, w, 0, True)["channel_splits"] > 1
     ref = oracle_layer(wt, bias, x, stride, storage, True)
-    for _ in range(3):   # the workspace must come back zeroed: repeated calls stay correct
-        y = layer.forward(xt, relu=True, split=True)
+    # the tiled kernel, whose path this is, and whatever a default call runs (the workspace must come back
+    # zeroed: repeated calls stay correct)
+    for kernel in (B.KERNEL_TILED,) * 3 + (0,) * 3:
+        y = layer.forward(xt, relu=True, kernel=kernel, split=True)
         torch.cuda.synchronize()
         check_close(y.float().cpu().numpy(), ref, storage, "split %s" % (case,))
-    assert not layer._ws.any()
+        assert not layer._ws.any()
     assert B.pconv_device_status(layer.handle)[0] == 0
     layer.close()
 
@@ -321,16 +324,17 @@ def test_reproducible_flag_gives_bit_identical_runs(case):
     xt = torch.from_numpy(x).cuda()
     ws = layer.workspace(xt.shape)
     ref = oracle_layer(wt, bias, x, stride, "f32", True)
-    first = None
-    for _ in range(6):
-        y = torch.empty(layer.out_shape(xt.shape), device="cuda")
-        B.pconv_forward(layer.handle, xt, layer.bias, y, B.RELU | B.REPRODUCIBLE, workspace=ws)
-        torch.cuda.synchronize()
-        got = y.cpu().numpy()
-        check_close(got, ref, "f32", "reproducible %s" % (case,))
-        if first is None:
-            first = got
-        assert np.array_equal(got, first)
+    for kernel in (B.KERNEL_TILED, 0):              # (a default call may run the dense kernel)
+        first = None
+        for _ in range(6):
+            y = torch.empty(layer.out_shape(xt.shape), device="cuda")
+            B.pconv_forward(layer.handle, xt, layer.bias, y, B.RELU | B.REPRODUCIBLE | kernel, workspace=ws)
+            torch.cuda.synchronize()
+            got = y.cpu().numpy()
+            check_close(got, ref, "f32", "reproducible %s" % (case,))
+            if first is None:
+                first = got
+            assert np.array_equal(got, first)
     if ws is not None:
         assert not ws.any()            # the flag keeps the channel range in one thread block
     assert B.pconv_device_status(layer.handle)[0] == 0
@@ -364,8 +368,8 @@ def test_every_warp_sharing_plan_matches_the_oracle():
             # planner's own choice does not split)
             assert plan["channel_splits"] == 1 or (with_ws and B.pconv_workspace_bytes(layer.handle, n, h, w) > 0)
             seen.add((plan["warps_per_unit"], plan["channel_splits"] > 1))
-            for _ in range(2):
-                y = layer.forward(xt, relu=True, split=with_ws)
+            for kernel in (B.KERNEL_TILED, B.KERNEL_TILED, 0):     # the plan is the tiled kernel's
+                y = layer.forward(xt, relu=True, kernel=kernel, split=with_ws)
                 torch.cuda.synchronize()
                 check_close(y.float().cpu().numpy(), ref, "f32", "plan %s of %s" % (plan, case))
         assert B.pconv_device_status(layer.handle)[0] == 0
