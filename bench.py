@@ -10,11 +10,12 @@ per GPU, fp32.
 A step is one pass of the whole stack over one image (per rank).  `value` is effective TFLOP/s
 (2 x surviving multiply-adds of all ranks / device time, inputs resident in HBM); `e2e` is the same
 figure through the host entry point (input copied from pinned host memory and the result copied
-back inside the timed region).  `configs` holds, for the other four benchmark configurations, the
+back inside the timed region).  `roofline` sets what the dense tensor-core kernel does for it (zero-inserted
+operations) against the measured bf16 rate, and the surviving operations against the FP32 pipe's peak.  `configs` holds, for the other four benchmark configurations, the
 time, effective TFLOP/s and roofline fraction of every layer.  `--impl reference` times the CPU
 oracle on the same workload.  Under torchrun every rank runs its own image (batch sharding, no
 collective on the data path).  `--layer` times one layer alone (the small case used for profiler
-captures) and prints its launch plan.
+captures) and prints the kernels that ran and the tiled kernel's launch plan.
 """
 import argparse
 import json
@@ -49,6 +50,42 @@ def hbm_peak_gbs():
             return float(json.load(f)["hbm_gbs"]), "measured (MEASURED_PEAKS.json)"
     except (OSError, KeyError, ValueError):
         return 6650.0, "fallback (earlier measurement on this pool)"
+
+
+def tensor_peak_tflops():
+    """(TFLOP/s, source): the measured burst bf16 GEMM rate of this machine's B200s, else the stated fallback."""
+    try:
+        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
+            return float(json.load(f)["bf16_tflops"]), "measured (MEASURED_PEAKS.json)"
+    except (OSError, KeyError, ValueError):
+        return 1590.0, "fallback (earlier measurement on this pool)"
+
+
+def config_of(world):
+    return {"workload": WORKLOAD, "images_per_step": world,
+            "l2": "flushed between timed steps on the device (256 MB write)",
+            "parallelism": "batch sharding, no collective"}
+
+
+def kernels_of(torch, fn):
+    """Names of this library's kernels that one call of fn() launches, in order (from torch's profiler; nothing
+    is timed here), or None where the profiler is not available."""
+    try:
+        from torch.profiler import ProfilerActivity, profile
+        torch.cuda.synchronize()
+        with profile(activities=[ProfilerActivity.CUDA]) as prof:
+            fn()
+            torch.cuda.synchronize()
+        events = sorted((e for e in prof.events() if "pconv" in e.name), key=lambda e: e.time_range.start)
+        names = [m.group(1) for m in (re.search(r"(\w+_kernel)\b", e.name) for e in events) if m]
+        return names or None
+    except Exception:
+        return None
+
+
+def dense_flops(spec, n=1, half=False):
+    """Operations of the dense kernel for a layer: every tap and channel, for fp32 six products of bf16 pieces."""
+    return 2.0 * 9 * spec.c_in * spec.c_out * spec.h_out * spec.w_out * n * (1 if half else 6)
 
 
 def recorded_traffic():
@@ -175,7 +212,7 @@ def run_reference(args):
         "impl": "reference", "metric": METRIC, "value": val, "unit": "TFLOP/s", "n_gpus": args.gpus,
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True,
         "scaling": "weak", "vs_baseline": None, "dtype": "f64", "data": "synthetic",
-        "config": {"workload": WORKLOAD, "images_per_step": 1},
+        "config": config_of(1),
         "ms_per_image": ms,
         "cpu_baseline": {"value": val, "unit": "TFLOP/s", "cores": cores, "kind": "oracle",
                          "sample": "whole stack (13 conv + 4 pool), 1 image per step, dense "
@@ -219,28 +256,19 @@ def measure_config(torch, B, flush, cid, batch, reps, hbm_gbs):
         pool = bool(cfg.chained and spec.pool_after)
         n_, c_, h_, w_ = layer.out_shape(x.shape)
         y = torch.empty((n_, c_, h_ // 2, w_ // 2) if pool else (n_, c_, h_, w_), dtype=tdtype, device="cuda")
-        plan = B.pconv_plan(layer.handle, cfg.batch, spec.h, spec.w, 0, True)
-        if pool and plan["tensor_path"]:
-            # what a stack launches here: the dense tensor-core kernel, then the plain max-pool kernel
-            y_full = torch.empty((n_, c_, h_, w_), dtype=tdtype, device="cuda")
 
-            def run(layer=layer, x=x, y=y, y_full=y_full):
-                layer.forward(x, relu=True, out=y_full, split=True)
-                B.pconv_maxpool2x2(y_full, y)
-        else:
-            def run(layer=layer, x=x, y=y, pool=pool):
-                layer.forward(x, relu=True, out=y, split=True, pool=pool)
+        def run(layer=layer, x=x, y=y, pool=pool):
+            layer.forward(x, relu=True, out=y, split=True, pool=pool)
         run()                                                          # warm-up (and the chain's data)
         us = _time_launch(torch, flush, run, reps)
         roof = layer_roof_us(spec, kept, cfg.batch, es, hbm_gbs)
         row = {"layer": spec.name, "us": round(us, 2), "roof_us": round(roof, 3),
                "frac": round(roof / us, 4),
                "tflops": round(layer_flops(spec, kept, cfg.batch) / us / 1e6, 3),
-               "kernel": "tensor" if plan["tensor_path"] else "tiled"}
-        if plan["tensor_path"]:
-            # the dense path's own roof: zero-inserted multiply-adds at the measured bf16 tensor peak
-            dense = 2.0 * 9 * spec.c_in * spec.c_out * spec.h_out * spec.w_out * cfg.batch
-            row["dense_tflops"] = round(dense / us / 1e6, 1)
+               "kernels": kernels_of(torch, run)}
+        if "dense_kernel" in (row["kernels"] or ()):
+            # what the tensor cores do for it: zero-inserted multiply-adds, for fp32 six products each
+            row["dense_tflops"] = round(dense_flops(spec, cfg.batch, half) / us / 1e6, 1)
         if cid == 5:
             s = layer.stats()
             mean = s.kept_kernels / max(s.n_groups, 1)
@@ -322,7 +350,8 @@ def run_layer(args):
         "layer": {"c_in": spec.c_in, "c_out": spec.c_out, "h": spec.h, "w": spec.w, "n": n,
                   "stride": spec.stride, "keep": spec.keep, "storage": storage,
                   "patterns": len(patterns), "kept_kernels": kept, "workspace": split},
-        "plan": B.pconv_plan(layer.handle, n, spec.h, spec.w, kflags, split),
+        "kernels": kernels_of(torch, lambda: layer.forward(x, out=y, split=split, kernel=kflags)),
+        "tiled_plan": B.pconv_plan(layer.handle, n, spec.h, spec.w, kflags, split),
         "us": round(us, 2), "tflops": round(layer_flops(spec, kept, n) / us / 1e6, 3),
         "frac_of_alu_peak": round(layer_flops(spec, kept, n) / us / 1e6 / ALU_PEAK_TFLOPS, 4),
         "roof_us": round(roof, 3), "frac": round(roof / us, 4), "hbm_peak": src,
@@ -425,7 +454,7 @@ def run_ours(args):
         raise SystemExit("device reported an abandoned wait in the chained stack")
     chain_stack.close()
 
-    # ---- per-kernel pass: the dominant kernel's launches timed one by one ------------------------
+    # ---- per-layer pass: the layers one by one, each from NCHW -------------------------------------
     acts = []
     a = x
     for layer, pool in zip(conv_layers, pools):
@@ -488,20 +517,24 @@ def run_ours(args):
         parity_ok = bool((err <= 1e-4 * (1 + np.abs(a_ref))).all())
         conv_time_ms = sum(conv_ms)
         roofs = [layer_roof_us(s, kept, 1, 4, hbm_gbs) for s, _, _, kept in layers]
-        # The timed region launches nothing but the 13 conv kernels (pools fused), so its duration
-        # is theirs, overlap between consecutive launches included; the launches timed one by one
-        # (no overlap) are reported beside it.
+        # The timed region launches nothing but the stack's kernels (one per layer, pools fused, and where position
+        # rows begin one that lays them out), so its duration is theirs, overlap between consecutive launches
+        # included; the layers run one by one (each from NCHW, no overlap) are reported beside it.
         achieved = flops / (ms_step * 1e-3) / 1e12
         achieved_alone = flops / (conv_time_ms * 1e-3) / 1e12
         value = world * flops / (ms_step * 1e-3) / 1e12
+        # which kernel ran which layer, and the operations the dense one did
+        launched = kernels_of(torch, lambda: stack.forward(x, y))
+        per_layer = [k for k in launched or [] if k in ("dense_kernel", "tiled_kernel")]
+        dense = sum(dense_flops(s) for (s, _, _, _), k in zip(layers, per_layer or ["dense_kernel"] * len(layers))
+                    if k == "dense_kernel") / (ms_step * 1e-3) / 1e12
+        tensor_peak, tensor_src = tensor_peak_tflops()
         out = {
             "metric": METRIC, "value": value, "unit": "TFLOP/s", "n_gpus": world,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms_step,
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f32",
             "data": "synthetic",
-            "config": {"workload": WORKLOAD, "images_per_step": world,
-                       "l2": "flushed between timed steps (256 MB write)",
-                       "parallelism": "batch sharding, no collective"},
+            "config": config_of(world),
             "ms_per_image": ms_step,
             "surviving_gflop_per_image": flops / 1e9,
             "roofline_time_us_per_image": sum(roofs),
@@ -509,7 +542,8 @@ def run_ours(args):
             "e2e": {"value": world * flops / (e2e_ms * 1e-3) / 1e12, "unit": "TFLOP/s",
                     "ms_per_step": e2e_ms, "h2d_bytes_per_step": int(x_host.numel() * 4),
                     "d2h_bytes_per_step": int(y_host.numel() * 4)},
-            # one launch per conv layer: the four max-pools are fused into the epilogue of the layer before
+            # one launch per conv layer (the four max-pools are fused into the epilogue of the layer before), and one
+            # more where a layer's input has to be laid out as position rows
             "gpu_launches": args.steps * stack.launches(),
             "graph_replay": {"ms_per_step": graph_ms, "value": flops / (graph_ms * 1e-3) / 1e12,
                              "unit": "TFLOP/s", "matches_eager_output": graph_same},
@@ -517,12 +551,16 @@ def run_ours(args):
             "chained": {"ms_per_step": chain_ms, "value": flops / (chain_ms * 1e-3) / 1e12,
                         "unit": "TFLOP/s", "launches_per_step": chain_launches,
                         "matches_eager_output": chain_same},
-            "roofline": {"bound": "alu", "kernel": "tiled_kernel (13 conv launches per step)",
-                         "achieved": achieved, "peak": ALU_PEAK_TFLOPS, "unit": "TFLOP/s",
-                         "frac": achieved / ALU_PEAK_TFLOPS,
-                         "peak_source": "148 SMs x 128 FP32 lanes x 2 x 1.965 GHz (derived; "
-                                        "no FP32 figure in MEASURED_PEAKS.json; an FFMA2 loop "
-                                        "measured 74.1, profiles/fp32_peak.md)",
+            # what bounds the step: the tensor pipe, on the dense kernel's zero-inserted operations; and beside it
+            # the surviving operations against the FP32 pipe's peak, which is the sparse kernel's roof
+            "roofline": {"bound": "tensor", "kernel": "dense_kernel", "launched": launched,
+                         "achieved": dense, "peak": tensor_peak, "unit": "TFLOP/s", "frac": dense / tensor_peak,
+                         "peak_source": "bf16 GEMM, " + tensor_src,
+                         "effective": achieved, "alu_peak": ALU_PEAK_TFLOPS,
+                         "effective_frac_of_alu_peak": achieved / ALU_PEAK_TFLOPS,
+                         "alu_peak_source": "148 SMs x 128 FP32 lanes x 2 x 1.965 GHz (derived; "
+                                            "no FP32 figure in MEASURED_PEAKS.json; an FFMA2 loop "
+                                            "measured 74.1, profiles/fp32_peak.md)",
                          "frac_of_layer_roofs": sum(roofs) / (ms_step * 1e3),
                          "hbm_peak_gbs": hbm_gbs, "hbm_peak_source": hbm_src,
                          "launch_ms_sum": conv_time_ms, "achieved_launches_timed_alone": achieved_alone,
