@@ -8,8 +8,10 @@
  * for weights that carry the two sparsities of the paper's "Sparse Convolution Pattern" section:
  * every surviving (filter o, input channel c) kernel has its non-zeros inside one 3x3 binary
  * pattern of a small set (pattern pruning: 4 of 9 taps, the "2.25x" of the pattern-count tables),
- * and whole kernels are removed (connectivity pruning).  The library skips every pruned kernel and
- * every tap outside the pattern; the result equals the dense convolution up to summation order.
+ * and whole kernels are removed (connectivity pruning).  The result is the sum over the surviving taps
+ * up to summation order: the sparse kernels skip every pruned kernel and every tap outside the
+ * pattern; the dense tensor-core kernel, taken where it is expected to be faster, multiplies zeros there
+ * and makes sure that nothing else comes of them (see PCONV_KERNEL_TENSOR).
  * Zero padding 1, stride 1 or 2, dilation 1, groups 1, optional bias and fused ReLU are fixed by
  * this build (the paper does not state them).
  *
@@ -59,15 +61,16 @@ enum {
   PCONV_RELU = 1u,    /* forward: y = max(0, .) after the bias */
   PCONV_STRICT4 = 2u, /* pack: every kernel must have exactly 0 or 4 non-zeros */
   PCONV_POOL2X2 = 4u, /* forward: a 2x2 / stride-2 max-pool is applied to the activated output in
-                         the same kernel (tiled kernels only); y then holds
+                         the same kernel (tiled and dense kernels); y then holds
                          [n][c_out][h_out/2][w_out/2] */
   /* Kernel selection (forward).  Default: the library picks per shape.  These bits exist so that
    * tests and benchmarks can pin one implementation; they never change the result beyond
    * summation order. */
   PCONV_REPRODUCIBLE = 8u, /* forward: the same call gives bit-identical outputs every time: the
-                              warps that share a tile take their chunks in a fixed order and the
-                              channel range is not split across thread blocks (a workspace, if
-                              given, is left untouched).  Without it the grouping of the fp32 partial
+                              warps that share a tile take their chunks in a fixed order, and a
+                              channel range is split across thread blocks only where they add
+                              their sums up in a fixed order (a workspace, if given, is left
+                              untouched).  Without it the grouping of the fp32 partial
                               sums -- not the result beyond rounding -- may vary from run to run. */
   PCONV_CHAIN = 0x10u,     /* stacks: consecutive layers whose launch plans are single waves of CTAs
                               (batch-1 inference) run as ONE persistent kernel: Tensor Memory,
@@ -78,7 +81,8 @@ enum {
                               faster (19 us per 512-filter 14x14 layer against 24 us chained). */
   PCONV_KERNEL_SIMPLE = 0x100u, /* one thread per output, walks the per-filter kernel list */
   PCONV_KERNEL_TILED = 0x200u,  /* shared-memory halo tiles, packed FMAs, one straight-line body per
-                                   pattern mask (any set of 4-of-9 masks); the default */
+                                   pattern mask (any set of 4-of-9 masks); the default where the dense
+                                   kernel is not expected to be faster */
   PCONV_KERNEL_GENERIC_TAPS = 0x400u, /* tiled path that tests the 9 mask bits at run time; slower,
                                          kept as a cross-check of the per-mask bodies */
   PCONV_ROWS4 = 0x1000u, /* tiled kernel with one-byte codes (canonical pattern sets): pins the */
@@ -114,7 +118,10 @@ enum {
                                   It multiplies the pruned zeros too -- 9 / (4 x keep rate) times the
                                   surviving multiply-adds, for fp32 storage six times that (three exact
                                   bf16 pieces a value, six products) -- and is still faster wherever
-                                  there is enough work for them, so the library picks it by estimate.
+                                  there is enough work for them, so a default forward picks it by
+                                  expected time, for both storage types, strides and with a fused pool.
+                                  The bit itself pins it for fp16 storage, stride 1, no pool only
+                                  (otherwise PCONV_ERR_UNSUPPORTED).
                                   fp16 products are exact in fp32; the fp32 form drops less than 2^-24 of
                                   a product, and its pieces are exact for activations and weights of
                                   magnitude 2^-110 up to the largest fp32 value (smaller ones to 2^-133).
@@ -174,13 +181,13 @@ pconv_status pconv_pack(const float* w_oihw_host, int c_out, int c_in, const uin
  *            layer's output is max-pooled before it is stored (the VGG stacks of the evaluation
  *            pool after conv2/4/7/10): y_dev is [n][c_out][h_out/2][w_out/2] (odd trailing row
  *            and column dropped, as pconv_maxpool2x2 does), h_out and w_out must be >= 2, and the
- *            call is refused with PCONV_ERR_UNSUPPORTED when no tiled kernel takes the shape or
- *            PCONV_KERNEL_SIMPLE is asked for.
+ *            call is refused with PCONV_ERR_UNSUPPORTED when neither the dense nor the tiled kernel
+ *            takes the shape or PCONV_KERNEL_SIMPLE is asked for.
  *
  * Asynchronous on `stream`; allocates nothing and never synchronises.  PCONV_ERR_CUDA reports
  * launch-time errors only.  A handle is immutable: concurrent forwards on several streams are
  * allowed.  n == 0 is a no-op.
- * The tiled kernels are launched with programmatic stream serialisation: a launch may begin its
+ * The tiled and dense kernels are launched with programmatic stream serialisation: a launch may begin its
  * own set-up while the previous kernel of the stream is still running, and waits for that kernel
  * to finish before it reads x or writes y, so stream order holds for every buffer named here.
  */
@@ -268,7 +275,7 @@ pconv_status pconv_maxpool2x2(const void* x_dev, void* y_dev, int n, int c, int 
  * (w_out: c_out*c_in*9 floats).  fp16 handles return the rounded values.  Synchronous. */
 pconv_status pconv_unpack(const pconv_handle* h, float* w_oihw_host_out);
 
-/* How the tiled kernel would run one forward (the paper has no counterpart: its tuning step picks
+/* How the tiled kernel would run one forward, whichever kernel a default call takes (the paper has no counterpart: its tuning step picks
  * tile sizes off line; here the library picks them per call from the shape). */
 typedef struct pconv_plan_t {
   int generic_taps;      /* 1 = run-time masks (asked for with PCONV_KERNEL_GENERIC_TAPS) */
@@ -288,8 +295,9 @@ typedef struct pconv_plan_t {
                             rebuilt into the kernel's tile layout by the producer warps */
   int tensor_path;       /* 1 = fp16 storage, stride 1, and a batch that gives the tensor cores enough
                             tiles: a default forward of this shape (no kernel-selection flag, no fused
-                            pool) runs the dense tensor-core kernel.  Other shapes run whichever kernel
-                            is estimated to be faster; the fields above still describe the tiled one */
+                            pool) runs the dense tensor-core kernel whatever is expected of it.  0 says
+                            nothing: other shapes, and all fp32 ones, run whichever kernel is expected
+                            to be faster.  The fields above describe the tiled kernel in either case */
 } pconv_plan_t;
 
 /* Test / tuning aid: fills *plan with the geometry a tiled forward of this shape would use;

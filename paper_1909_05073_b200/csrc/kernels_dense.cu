@@ -7,7 +7,7 @@
 // of which the sparse kernel's per-kernel jump leaves 15-20.
 //
 // Precision.  fp16 storage: products are exact in fp32, sums are fp32.  fp32 storage: every activation
-// and weight is cut into three bf16 pieces, x = x1 + x2 + x3 exactly (8 + 8 + 8 bits, rounded to nearest
+// and weight is cut into three bf16 pieces, x = x1 + x2 + x3 exactly (from 2^-110 up; 8 + 8 + 8 bits, rounded to nearest
 // so that the pieces' signs are random), and six of the nine piece products are formed:
 //   main  x1 w1;   cross  x1 w2, x2 w1, x2 w2, x1 w3, x3 w1
 // The three left out are below 2^-24 of the product together.  The tensor core adds with truncation
@@ -47,7 +47,7 @@
 //    epilogue unrolled over its registers took 10 us a tile to fetch, a wait loop unrolled by the compiler
 //    half of the kernel's speed.
 //  * What bounds it: the tensor pipe in large fp32 launches (512->512 14x14 N=64: 589 us in the sparse
-//    kernel, 326 here); with 64 filters or few channels the epilogue; at one image a fixed 9-10 us of
+//    kernel, 312 here); with 64 filters or few channels the epilogue; at one image a fixed 9-10 us of
 //    launch, first copies and exchange, then the weight stream (36 bytes a cycle and SM from L2).
 //  * Every wait is bounded; one that runs out records its id in the status word, the role stops
 //    working, and all roles meet at the common exit where Tensor Memory is released.
@@ -2112,9 +2112,9 @@ cudaError_t launch_dense(const DeviceLayer& L, const void* x, const float* bias,
 
 // What is expected to run this shape fastest: both kernels by estimate.  Sparse kernel: a fixed 12 us, 8 ns a
 // channel, twice that at stride 2 (measured at 1 image: 14-15 us at 64-128 channels, 18-23 us at 512) and a
-// fifth of the FP32 peak (15-29 % of it in large launches).  Dense kernel: measured times are 1.3-1.45 times
-// the estimated cycles at the full clock, of which the clock under tensor load (1.65 of 1.9 GHz) is the larger
-// part.  Staging the input as position rows is a launch of its own and moves every value twice.  Where a
+// fifth of the FP32 peak (15-29 % of it in large launches).  Dense kernel: its plan's cycles at 1380 a microsecond,
+// which is coarse: 1113 fp32 chains of equal layers took 0.97-1.76 of that (5th to 95th percentile, median
+// 1.32; 1.5 at 32 filters a tile, 1.0 at 128), the stress layers of 64 images 1.08 (stride 1) and 1.22.  Staging the input as position rows is a launch of its own and moves every value twice.  Where a
 // tile's positions are all there are, each dense weight (54 bytes for fp32, a kept kernel's sparse ones take 6
 // a weight) is read for one use and, in a network of such layers, from memory: 512->512 7x7 takes 15 us alone
 // and 20-26 us among its neighbours, the sparse kernel 18 us in both.

@@ -3,7 +3,9 @@
 // per kernel the pattern that retains the largest sum of squares; the k-th largest retained sum by a
 // radix select on the bits of the (non-negative) fp32 sums, 11 + 11 + 10 bits; masking.
 //
-// Bound by memory: the weights are read twice (the second time partly from L2) and written once.  Five
+// The weights are read twice (the second time partly from L2) and written once: 35 us at the copy rate for
+// 4096x512 kernels, of which it takes 101 us -- scoring 35, masking 35, digits 24, ids 7.  What the scoring and
+// masking passes spend the rest on has not been shown; ~200 instructions a kernel are 11 us of issue.  Five
 // launches: the first digit's histogram is taken where the sums are formed, and the block that finishes a
 // histogram last picks the digit, so no launch exists for the picks.
 #include <algorithm>
