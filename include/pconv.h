@@ -128,7 +128,8 @@ enum {
                                   A result differs from the sparse kernels' by summation order only: an
                                   infinite activation or a NaN reaches the outputs that have it under a
                                   surviving tap and no others.  (Outputs whose dense sum is not finite are
-                                  formed again from the surviving taps, at the speed of the plain kernel.) */
+                                  formed again from the surviving taps, at the speed of the plain kernel: up to
+                                  150 times the usual time where infinities are everywhere.) */
 };
 
 #define PCONV_MAX_PATTERNS 16
